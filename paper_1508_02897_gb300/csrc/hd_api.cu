@@ -97,6 +97,7 @@ static void free_ctx(hd_ctx *c) {
   if (c->d_gay_c) cudaFreeAsync(c->d_gay_c, c->stream);
   if (c->d_giay_f) cudaFreeAsync(c->d_giay_f, c->stream);
   if (c->d_lpool) cudaFreeAsync(c->d_lpool, c->stream);
+  if (c->d_lpoolf) cudaFreeAsync(c->d_lpoolf, c->stream);
   if (c->d_subs) cudaFreeAsync(c->d_subs, c->stream);
   if (c->d_axx) cudaFreeAsync(c->d_axx, c->stream);
   if (c->d_axy) cudaFreeAsync(c->d_axy, c->stream);
@@ -235,6 +236,7 @@ int hd_setup_medium(hd_ctx **out, const hd_grid *grid, const hd_decomp *dec, con
   ALLOC(c->d_gay_c, sizeof(double2) * c->NY);
   ALLOC(c->d_giay_f, sizeof(double2) * (c->NY + 1));
   ALLOC(c->d_lpool, sizeof(double2) * aoff);
+  ALLOC(c->d_lpoolf, sizeof(float2) * aoff);
   ALLOC(c->d_subs, sizeof(SubDev) * c->nsub);
   ALLOC(c->d_axx, sizeof(AxisDev) * c->nbx);
   ALLOC(c->d_axy, sizeof(AxisDev) * c->nby);

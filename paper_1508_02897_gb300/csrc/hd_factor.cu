@@ -148,7 +148,8 @@ k_factor(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, cons
           for (int I = 0; I <= J; ++I, ++u) {
             const S *tile = prev + (int64_t)u * 256;
             {
-              const int cc = tid >> 4, rr = ((tid & 15) - cc) & 15;   // storage order
+              int rr, cc;   // storage order
+              sym_entry<S>(tid, rr, cc);
               const int r = 16 * I + rr, c = 16 * J + cc;
               if (r < m && c < m)
                 W[(int64_t)c * m + r] = cfms(cmul(lS[r], load_c<T>(tile[tid])), lS[c],
@@ -158,7 +159,7 @@ k_factor(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, cons
               const int rr = tid >> 4, cc = tid & 15;   // W(16J + cc, 16I + rr) = S(16I + rr, 16J + cc)
               const int r = 16 * J + cc, c = 16 * I + rr;
               if (r < m && c < m)
-                W[(int64_t)c * m + r] = cfms(cmul(lS[r], load_c<T>(tile[cc * 16 + ((rr + cc) & 15)])), lS[c],
+                W[(int64_t)c * m + r] = cfms(cmul(lS[r], load_c<T>(tile[sym_pos<S>(rr, cc)])), lS[c],
                                              d_band<T, R>(r, c, j, a1c, ia1f, a2c, ia2f, k2row, h2));
             }
           }
@@ -328,11 +329,12 @@ k_factor(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, cons
       __syncthreads();
       if (SYM) {
         // upper 16 x 16 tiles (I, J), I <= J, of the exactly symmetric matrix
-        // S^{-1}[min(r,c)][max(r,c)]: tile at J(J+1)/2 + I, entry (r, c) at c*16 + ((r + c) & 15)
+        // S^{-1}[min(r,c)][max(r,c)]: tile at J(J+1)/2 + I, entries placed by sym_pos
         S *tiles = slot + (int64_t)(J * (J + 1) / 2) * 256;
         for (int e2 = tid; e2 < (J + 1) * 256; e2 += FT) {
           const int I = e2 >> 8, e = e2 & 255;
-          const int cc = e >> 4, rr = ((e & 15) - cc) & 15;
+          int rr, cc;
+          sym_entry<S>(e, rr, cc);
           const int r = I * 16 + rr, c = c0 + cc;
           T v = mk<T>(0, 0);
           if (r < m && c < m) v = r <= c ? Q[cc * m + r] : Q[(r - c0) * m + c];

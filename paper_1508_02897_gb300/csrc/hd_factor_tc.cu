@@ -567,8 +567,8 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
                   for (int i = 0; i < 16; ++i) {
                     const int c = c0 + i;
                     const float2 v = (r < m && c < m) ? make_float2(re[i], im[i]) : make_float2(0.f, 0.f);
-                    if (J > I || i >= rr) tile[i * 16 + ((rr + i) & 15)] = store_c<S>(v);
-                    if (J == I && i > rr) tile[rr * 16 + ((i + rr) & 15)] = store_c<S>(v);
+                    if (J > I || i >= rr) tile[sym_pos<S>(rr, i)] = store_c<S>(v);
+                    if (J == I && i > rr) tile[sym_pos<S>(i, rr)] = store_c<S>(v);
                   }
                 }
               } else {

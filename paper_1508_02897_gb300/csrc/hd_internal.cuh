@@ -94,6 +94,20 @@ __device__ __forceinline__ float2 ds_split(double x) {
   const float l0 = __fsub_rn(__uint_as_float(e0 | (lo & 63u)), __uint_as_float(e0));
   return make_float2(h, __fadd_rn(l1, l0));
 }
+// FP64 -> FP32, rounded to nearest even like the conversion instruction but on the integer
+// pipe: the 29 dropped bits round through a carry into the kept ones.  Exponents whose
+// result could be subnormal or overflow (and zero, inf, NaN) take the instruction.
+__device__ __forceinline__ float d2f_rn(double x) {
+  const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
+  const unsigned int e = (hi >> 20) & 0x7FFu;
+  if (e - 897u > 1149u - 897u) return (hi << 1 | lo) == 0u ? __uint_as_float(hi) : __double2float_rn(x);
+  const unsigned int t = __funnelshift_l(lo, hi, 3);   // low 32 bits of the kept field and below
+  const unsigned int r = ((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (t & 1u)) >> 29;
+  return __uint_as_float((hi & 0x80000000u) | ((((e - 896u) << 23) | (t & 0x7FFFFFu)) + r));
+}
+template <typename R> __device__ __forceinline__ R from_d(double x);
+template <> __device__ __forceinline__ float from_d<float>(double x) { return d2f_rn(x); }
+template <> __device__ __forceinline__ double from_d<double>(double x) { return x; }
 // float -> FP64 by moving the fields (exact); zero gives 0, subnormals, inf and NaN convert.
 __device__ __forceinline__ double ds_f2d(float f) {
   const unsigned int u = __float_as_uint(f);
@@ -188,6 +202,58 @@ __device__ __forceinline__ T d_band(int r, int c, int j, const double2 *a1c, con
 // imaginary lo), hi = TF32 rounding and lo = TF32 rounding of the remainder (HD_TF32X3).
 enum { LAY_FULL = 0, LAY_SYM = 1, LAY_TC = 2, LAY_TC3 = 3 };
 
+// Symmetric tile storage: the upper 16 x 16 tiles of an m x m block, column by column
+// (tile (I, J) at J(J+1)/2 + I, I <= J < mt = ceil(m / 16)).  The substitution takes them in
+// segments: up to SYM_SEG tiles one above the other, (3k .. 3k + 2, J); segments are numbered
+// column by column and cut into SYM_GROUPS groups of consecutive ones, whose sums are formed
+// apart (SymMap: the numbering, shared by the kernel and its tables).
+constexpr int SYM_SEG = 3, SYM_GROUPS = 4;
+struct SymMap {
+  int mt, nt, nseg, base, rem;
+  __host__ __device__ explicit SymMap(int m) {
+    mt = (m + 15) / 16;
+    nt = mt * (mt + 1) / 2;
+    nseg = col_seg(mt);
+    base = nseg / SYM_GROUPS;
+    rem = nseg - base * SYM_GROUPS;
+  }
+  // first segment of column J: the columns before it have 1, 1, 1, 2, 2, 2, 3, ... segments
+  static __host__ __device__ int col_seg(int J) {
+    const int q = J / SYM_SEG, r = J - q * SYM_SEG;
+    return SYM_SEG * q * (q + 1) / 2 + r * (q + 1);
+  }
+  __host__ __device__ int group_start(int g) const { return g * base + (g < rem ? g : rem); }   // in segments
+  __host__ __device__ int group_of(int s) const {
+    const int big = rem * (base + 1);
+    return s < big ? s / (base + 1) : rem + (s - big) / base;
+  }
+  // first tile and column of segment s (s = nseg: one past the last tile)
+  __host__ __device__ void segment(int s, int &I, int &J) const {
+    J = 0;
+    while (J < mt && col_seg(J + 1) <= s) ++J;
+    I = SYM_SEG * (s - col_seg(J));
+  }
+  __host__ __device__ int first_tile(int s) const {
+    int I, J;
+    segment(s, I, J);
+    return J * (J + 1) / 2 + I;
+  }
+};
+// Place of entry (r, c) in a tile: lane 8 (c / 4) + r / 2 of a warp holds rows 2 (r / 2) + e and
+// columns 4 (c / 4) + q; entries of one (q, e) lie side by side over the lanes (16-byte
+// entries) or as (e = 0, 1) pairs (narrower ones: one load of up to 16 bytes per lane).
+// Both keep 16 rows of a column together, and the warp's reads free of bank conflicts.
+template <typename S> __host__ __device__ __forceinline__ int sym_pos(int r, int c) {
+  const int lane = (c >> 2) * 8 + (r >> 1), q = c & 3, e = r & 1;
+  return sizeof(S) == 16 ? (q * 2 + e) * 32 + lane : q * 64 + lane * 2 + e;
+}
+// Row and column of place k (the inverse of sym_pos).
+template <typename S> __host__ __device__ __forceinline__ void sym_entry(int k, int &r, int &c) {
+  const int q = k >> 6, lane = sizeof(S) == 16 ? k & 31 : (k >> 1) & 31, e = sizeof(S) == 16 ? (k >> 5) & 1 : k & 1;
+  r = 2 * (lane & 7) + e;
+  c = 4 * (lane >> 3) + q;
+}
+
 __device__ __forceinline__ float tf32_round(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -258,6 +324,7 @@ struct hd_ctx {
   double *d_cc = nullptr;   // h^2 k^2 - 4: the centre coefficient of A outside the PML
   double2 *d_gax_c = nullptr, *d_giax_f = nullptr, *d_gay_c = nullptr, *d_giay_f = nullptr;
   double2 *d_lpool = nullptr;   // per-box PML tables: a1c[ex], ia1f[ex+1], a2c[ey], ia2f[ey+1]
+  float2 *d_lpoolf = nullptr;   // the same rounded to FP32
   hd::SubDev *d_subs = nullptr;
   hd::AxisDev *d_axx = nullptr, *d_axy = nullptr;
   int32_t *d_nearx = nullptr, *d_neary = nullptr;  // per global index: box column/row nearest
@@ -329,6 +396,10 @@ int run_apply_steps(hd_ctx *ctx, const double2 *r, int64_t rs, double2 *z, int64
 // r = b - A x with strided vectors (nrhs on grid.z)
 cudaError_t launch_residual_strided(hd_ctx *ctx, const double2 *b, int64_t bs, const double2 *x, int64_t xs,
                                     double2 *r, int64_t rs, int nrhs, cudaStream_t st);
+// Restrict + forward/back substitution over the symmetric tile storage (hd_subst_sym.cu), staging out.
+cudaError_t launch_subst_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
+                             int64_t stg_stride, cudaStream_t st);
+int subst_sym_threads(const hd_ctx *ctx);
 // Restrict + forward/back substitution on the tensor cores (HD_TCORE storage), staging out.
 cudaError_t launch_subst_tc(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
                             int64_t stg_stride, cudaStream_t st);

@@ -41,7 +41,7 @@ __global__ void k_global_tables(double2 *ax_c, double2 *iax_f, double2 *ay_c, do
 }
 
 // Per box: the PML of Omega_ij itself (its outer npml cells on every side).
-__global__ void k_local_tables(const SubDev *subs, double2 *pool, int npml, double s0, int power) {
+__global__ void k_local_tables(const SubDev *subs, double2 *pool, float2 *poolf, int npml, double s0, int power) {
   const SubDev s = subs[blockIdx.x];
   double2 *a1c = pool + s.aoff;
   double2 *ia1f = a1c + s.ex;
@@ -49,6 +49,9 @@ __global__ void k_local_tables(const SubDev *subs, double2 *pool, int npml, doub
   double2 *ia2f = a2c + s.ey;
   fill_segment(a1c, ia1f, s.ex, npml, s0, power, threadIdx.x, blockDim.x);
   fill_segment(a2c, ia2f, s.ey, npml, s0, power, threadIdx.x, blockDim.x);
+  __syncthreads();
+  for (int i = threadIdx.x; i < 2 * s.ex + 2 * s.ey + 2; i += blockDim.x)
+    poolf[s.aoff + i] = make_float2((float)a1c[i].x, (float)a1c[i].y);
 }
 
 // k^2 = (omega / c)^2 per cell, and the centre coefficient h^2 k^2 - 4 that A has
@@ -68,7 +71,7 @@ __global__ void k_wavenumber(const double *__restrict__ c, double *__restrict__ 
 cudaError_t launch_setup_tables(hd_ctx *ctx, const double *c_dev, cudaStream_t st) {
   k_global_tables<<<2, 256, 0, st>>>(ctx->d_gax_c, ctx->d_giax_f, ctx->d_gay_c, ctx->d_giay_f, ctx->NX, ctx->NY,
                                      ctx->npml, ctx->s0, ctx->power);
-  k_local_tables<<<ctx->nsub, 256, 0, st>>>(ctx->d_subs, ctx->d_lpool, ctx->npml, ctx->s0, ctx->power);
+  k_local_tables<<<ctx->nsub, 256, 0, st>>>(ctx->d_subs, ctx->d_lpool, ctx->d_lpoolf, ctx->npml, ctx->s0, ctx->power);
   int64_t n = (int64_t)ctx->NX * ctx->NY;
   k_wavenumber<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(c_dev, ctx->d_k2, ctx->d_cc, n, ctx->omega,
                                                              ctx->h * ctx->h, ctx->d_status);

@@ -298,242 +298,6 @@ k_subst(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, const
   }
 }
 
-// ---------------------------------------------------------------------------
-// Symmetric storage.  A is complex symmetric, so every S_j and S_j^{-1} is too,
-// and only the upper 16 x 16 tiles of S_j^{-1} are stored: tile (I, J), I <= J,
-// at position J(J+1)/2 + I, entry (r, c) of a tile at c*16 + ((r + c) & 15)
-// (the rotation keeps row- and column-wise reads free of bank conflicts).
-// This streams about (mt+1)/(2 mt) of the bytes of the full blocks.  A tile
-// (I, J) serves twice: y_I += T v_J and, off the diagonal, y_J += T^T v_I.
-// A ring stage holds NW * TPW consecutive tiles and every consumer warp takes
-// TPW of them (tile du of a stage belongs to warp du % NW), so all warps work
-// on every stage.  In a warp, lane (rr, h) covers row / column rr of the tile
-// and the terms of parity h; after one shuffle the h = 0 lanes add the row-wise
-// sums and the h = 1 lanes the column-wise sums into the warp's own partial
-// vector in shared memory, and the step ends with y[a] = sum over warps of the
-// partials (a fixed order: results do not depend on timing).
-constexpr int TB = 16;
-
-template <typename S> __host__ __device__ constexpr int sym_tiles_per_warp() {
-  return sizeof(S) == 16 ? 1 : (sizeof(S) == 8 ? 1 : 2);
-}
-
-template <typename T, typename S>
-__host__ __device__ inline size_t subst_sym_smem(int ns, int mp, int nw, int nr, int nt) {
-  size_t o = (size_t)ns * nw * sym_tiles_per_warp<S>() * TB * TB * sizeof(S);
-  o += (size_t)nr * mp * sizeof(T) + (size_t)nw * nr * mp * sizeof(T);
-  o += 2 * (size_t)nt;
-  o = (o + 15) & ~(size_t)15;
-  return o + 2 * (size_t)ns * sizeof(uint64_t) + 16;
-}
-
-template <typename R, typename S, int NW, int NR>
-__global__ void __launch_bounds__(NW * 32 + 32)
-k_subst_sym(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, const S *__restrict__ factor,
-            const double2 *__restrict__ rg, int NX, int64_t vec_stride, C<R> *__restrict__ staging,
-            int64_t stg_stride, int nrhs, int NS, int mpmax, int32_t *status) {
-  using T = C<R>;
-  constexpr int CT = NW * 32;
-  constexpr int TPW = sym_tiles_per_warp<S>();
-  constexpr int TPC = NW * TPW;   // tiles per ring stage
-  constexpr int TE = TB * TB;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const SubDev s = subs[blockIdx.y];
-  const int m = s.ex, rows = s.ey;
-  const int mt = (m + TB - 1) / TB, mp = mt * TB, nt = mt * (mt + 1) / 2;
-  const int ntmax = (mpmax / TB) * (mpmax / TB + 1) / 2;
-  const int r0 = blockIdx.x * NR;
-  S *ring = reinterpret_cast<S *>(smem_raw);
-  T *vs = reinterpret_cast<T *>(ring + (size_t)NS * TPC * TE);   // [NR][mpmax]
-  T *part = vs + (size_t)NR * mpmax;                               // [NW][NR][mpmax]
-  uint8_t *tI = reinterpret_cast<uint8_t *>(part + (size_t)NW * NR * mpmax);
-  uint8_t *tJ = tI + ntmax;
-  size_t off = (size_t)NS * TPC * TE * sizeof(S) + (size_t)(NW + 1) * NR * mpmax * sizeof(T) + 2 * (size_t)ntmax;
-  off = (off + 15) & ~(size_t)15;
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + off);
-  uint64_t *empty = full + NS;
-  volatile int *abort_flag = reinterpret_cast<volatile int *>(empty + NS);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) {
-    for (int q = 0; q < NS; ++q) {
-      mbar_init(&full[q], 1);
-      mbar_init(&empty[q], NW);
-    }
-    *abort_flag = 0;
-    mbar_fence_init();
-  }
-  for (int J = 0; J < mt; ++J)
-    for (int I = tid; I <= J; I += blockDim.x) {
-      tI[J * (J + 1) / 2 + I] = (uint8_t)I;
-      tJ[J * (J + 1) / 2 + I] = (uint8_t)J;
-    }
-  for (int i = tid; i < NW * NR * mpmax; i += blockDim.x) part[i] = mk<T>(0, 0);
-  __syncthreads();
-
-  const int nck = (nt + TPC - 1) / TPC;
-  const int64_t total = (int64_t)(2 * rows - 1) * nck;
-  const int64_t slot_elems = (int64_t)nt * TE;
-  const S *Fs = factor + s.foff;
-
-  if (warp == NW) {
-    // ---------------- producer warp: stream the tiles in use order
-    if (lane == 0) {
-      int64_t issued = 0;
-      bool ok = true;
-      for (int64_t it = 0; it < total && ok; ++it) {
-        const int st = (int)(it / nck), c = (int)(it - (int64_t)st * nck);
-        const int j = st < rows ? st : 2 * rows - 2 - st;
-        const int slot = (int)(it % NS);
-        const uint32_t ph = (uint32_t)((it / NS) & 1);
-        if (!mbar_wait(&empty[slot], ph ^ 1u, abort_flag)) { ok = false; break; }
-        const int ntile = min(TPC, nt - c * TPC);
-        const uint32_t bytes = (uint32_t)(ntile * TE * sizeof(S));
-        mbar_arrive_expect_tx(&full[slot], bytes);
-        bulk_g2s(ring + (size_t)slot * TPC * TE, Fs + j * slot_elems + (int64_t)c * TPC * TE, bytes, &full[slot]);
-        issued = it + 1;
-      }
-      if (!ok) {
-        *abort_flag = 1;
-        atomicOr(status, ST_TIMEOUT);
-      }
-      for (int64_t it = max((int64_t)0, issued - NS); it < issued; ++it)
-        mbar_wait(&full[it % NS], (uint32_t)((it / NS) & 1), abort_flag);
-    }
-    return;
-  }
-
-  // ---------------- consumer warps (thread a owns output a of the step, a < mp)
-  const double2 *a1c = pool + s.aoff;
-  const double2 *a2c = a1c + 2 * m + 1;
-  const double2 *ia2f = a2c + rows;
-  const int a = tid;
-  const int gx = s.ex0 + a;
-  const bool ownx = a < m && gx >= s.ox0 && gx < s.ox1;
-  T a1 = mk<T>(0, 0);
-  if (a < m) {
-    const double2 t = a1c[a];
-    a1 = mk<T>((R)t.x, (R)t.y);
-  }
-  T w[NR];
-#pragma unroll
-  for (int q = 0; q < NR; ++q) w[q] = mk<T>(0, 0);
-  const int rr = lane & 15, h = lane >> 4;
-  int64_t it = 0;
-  bool ok = true;
-  for (int st = 0; st < 2 * rows - 1; ++st) {
-    const bool fwd = st < rows;
-    const int j = fwd ? st : 2 * rows - 2 - st;
-    consumer_sync(CT);   // the previous step's reads of vs are done
-    if (a < mp) {
-      if (fwd) {
-        const int gy = s.ey0 + j;
-        const bool owny = gy >= s.oy0 && gy < s.oy1;
-        const double2 isd = ia2f[j];
-        const T la = cmul(a1, mk<T>((R)isd.x, (R)isd.y));
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          T rho = mk<T>(0, 0);
-          if (owny && ownx && r0 + q < nrhs) {
-            const double2 rv = rg[(int64_t)(r0 + q) * vec_stride + (int64_t)gy * NX + gx];
-            rho = mk<T>((R)rv.x, (R)rv.y);
-          }
-          vs[q * mpmax + a] = a < m ? (j > 0 ? cfms(la, w[q], rho) : rho) : mk<T>(0, 0);
-        }
-      } else {
-        const double2 ind = ia2f[j + 1];
-        const T ua = cmul(a1, mk<T>((R)ind.x, (R)ind.y));
-#pragma unroll
-        for (int q = 0; q < NR; ++q) vs[q * mpmax + a] = a < m ? cmul(ua, w[q]) : mk<T>(0, 0);
-      }
-    }
-    consumer_sync(CT);
-    T *pw = part + (size_t)warp * NR * mpmax;
-    for (int c = 0; c < nck; ++c, ++it) {
-      const int slot = (int)(it % NS);
-      if (ok && !mbar_wait(&full[slot], (uint32_t)((it / NS) & 1), abort_flag)) {
-        ok = false;
-        *abort_flag = 1;
-        atomicOr(status, ST_TIMEOUT);
-      }
-      const S *stage = ring + (size_t)slot * TPC * TE;
-      const int u0 = c * TPC;
-#pragma unroll
-      for (int t = 0; t < TPW; ++t) {
-        const int du = t * NW + warp;
-        if (u0 + du >= nt) break;
-        const int I = tI[u0 + du], J = tJ[u0 + du];
-        const S *tile = stage + du * TE;
-        T pr[NR], pc[NR];
-#pragma unroll
-        for (int q = 0; q < NR; ++q) { pr[q] = mk<T>(0, 0); pc[q] = mk<T>(0, 0); }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int cc = 2 * k + h;   // halves interleaved: conflict-free for 4- and 8-byte entries
-          const T tv = load_c<T>(tile[cc * TB + ((rr + cc) & 15)]);   // T[rr][cc]
-#pragma unroll
-          for (int q = 0; q < NR; ++q) pr[q] = cfma(tv, vs[q * mpmax + J * TB + cc], pr[q]);
-        }
-        if (I != J) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int ai = 2 * k + h;
-            const T tv = load_c<T>(tile[rr * TB + ((ai + rr) & 15)]);  // T[ai][rr]
-#pragma unroll
-            for (int q = 0; q < NR; ++q) pc[q] = cfma(tv, vs[q * mpmax + I * TB + ai], pc[q]);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          pr[q].x += __shfl_xor_sync(0xffffffffu, pr[q].x, 16);
-          pr[q].y += __shfl_xor_sync(0xffffffffu, pr[q].y, 16);
-          pc[q].x += __shfl_xor_sync(0xffffffffu, pc[q].x, 16);
-          pc[q].y += __shfl_xor_sync(0xffffffffu, pc[q].y, 16);
-        }
-        if (h == 0) {
-#pragma unroll
-          for (int q = 0; q < NR; ++q) {
-            T *dst = pw + q * mpmax + I * TB + rr;
-            *dst = cadd(*dst, pr[q]);
-          }
-        } else if (I != J) {
-#pragma unroll
-          for (int q = 0; q < NR; ++q) {
-            T *dst = pw + q * mpmax + J * TB + rr;
-            *dst = cadd(*dst, pc[q]);
-          }
-        }
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[slot]);
-    }
-    consumer_sync(CT);   // every warp's partial sums are in shared memory
-    if (a < m) {
-#pragma unroll
-      for (int q = 0; q < NR; ++q) {
-        T y = mk<T>(0, 0);
-        for (int ww = 0; ww < NW; ++ww) {
-          T *p = part + ((size_t)ww * NR + q) * mpmax + a;
-          y = cadd(y, *p);
-          *p = mk<T>(0, 0);
-        }
-        if (r0 + q < nrhs) {
-          T *stg = staging + (int64_t)(r0 + q) * stg_stride + s.soff;
-          if (fwd) {
-            w[q] = y;
-            stg[(int64_t)j * m + a] = y;
-          } else {
-            const T x = csub(stg[(int64_t)j * m + a], y);
-            w[q] = x;
-            stg[(int64_t)j * m + a] = x;
-          }
-        } else {
-          w[q] = y;
-        }
-      }
-    }
-  }
-}
-
 // One axis of the smoothing function beta_ij (Remark after Eq. (pc)) at cell x of a box
 // [e0, e1) owning [o0, o1): 1 on the owned cells, else the C^2 step
 // S(t) = t^3 (10 - 15 t + 6 t^2) of t = 1 - d / (W + 1), d the distance from the owned
@@ -706,43 +470,6 @@ static cudaError_t launch_subst_nr(hd_ctx *ctx, const double2 *r, int nrhs, int6
   }
 }
 
-template <typename R, typename S, int NW, int NR>
-static cudaError_t launch_subst_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
-                                    int64_t stg_stride, cudaStream_t st) {
-  using T = C<R>;
-  const int mpmax = (ctx->max_m + TB - 1) / TB * TB;
-  const int ntmax = (mpmax / TB) * (mpmax / TB + 1) / 2;
-  const int groups = (nrhs + NR - 1) / NR;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int per_sm = (int)std::min<int64_t>(7, ((int64_t)ctx->nsub * groups + sms - 1) / sms);
-  const size_t fixed = subst_sym_smem<T, S>(0, mpmax, NW, NR, ntmax);
-  const size_t stage = (size_t)NW * sym_tiles_per_warp<S>() * TB * TB * sizeof(S);
-  const size_t budget = (size_t)200 * 1024 / (size_t)std::max(1, per_sm);
-  int ns = ctx->tune_ns > 0 && NR == 1 ? ctx->tune_ns : (budget > fixed ? (int)((budget - fixed) / (stage + 16)) : 2);
-  ns = std::min(32, std::max(2, ns));
-  const size_t smem = subst_sym_smem<T, S>(ns, mpmax, NW, NR, ntmax);
-  cudaError_t e = allow_smem(k_subst_sym<R, S, NW, NR>, smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(groups, ctx->nsub);   // a box's source groups run side by side and share its factor reads in L2
-  k_subst_sym<R, S, NW, NR><<<grid, NW * 32 + 32, smem, st>>>(ctx->d_subs, ctx->d_lpool,
-                                                              reinterpret_cast<const S *>(ctx->factor), r, ctx->NX,
-                                                              vec_stride, reinterpret_cast<T *>(staging), stg_stride,
-                                                              nrhs, ns, mpmax, ctx->d_status);
-  return cudaGetLastError();
-}
-
-template <typename R, typename S, int NW>
-static cudaError_t launch_subst_sym_nr(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
-                                       cudaStream_t st) {
-  switch (rhs_per_cta(nrhs)) {
-    case 8: return launch_subst_sym<R, S, NW, 8>(ctx, r, nrhs, vs, stg, ss, st);
-    case 4: return launch_subst_sym<R, S, NW, 4>(ctx, r, nrhs, vs, stg, ss, st);
-    case 2: return launch_subst_sym<R, S, NW, 2>(ctx, r, nrhs, vs, stg, ss, st);
-    default: return launch_subst_sym<R, S, NW, 1>(ctx, r, nrhs, vs, stg, ss, st);
-  }
-}
-
 template <typename R, typename S>
 static cudaError_t launch_apply_r(hd_ctx *ctx, const double2 *r, int64_t rs, double2 *z, int64_t zs, int nrhs,
                                   void *staging, cudaStream_t st) {
@@ -750,9 +477,7 @@ static cudaError_t launch_apply_r(hd_ctx *ctx, const double2 *r, int64_t rs, dou
     tic(ctx, T_SUBST, st);
     cudaError_t e = ctx->tc3  ? launch_subst_x3(ctx, r, nrhs, rs, staging, ctx->staging_elems, st)
                     : ctx->tc ? launch_subst_tc(ctx, r, nrhs, rs, staging, ctx->staging_elems, st)
-                    : (ctx->max_m <= 192 && ctx->tune_ct != 256)
-                        ? launch_subst_sym_nr<R, S, 6>(ctx, r, nrhs, rs, staging, ctx->staging_elems, st)
-                        : launch_subst_sym_nr<R, S, 8>(ctx, r, nrhs, rs, staging, ctx->staging_elems, st);
+                              : launch_subst_sym(ctx, r, nrhs, rs, staging, ctx->staging_elems, st);
     toc(ctx, T_SUBST, st, 1);
     if (e != cudaSuccess) return e;
     dim3 grid((ctx->NX + 255) / 256, (ctx->NY + GR - 1) / GR, nrhs);
@@ -831,7 +556,7 @@ int run_apply_steps(hd_ctx *ctx, const double2 *r, int64_t rs, double2 *z, int64
 }  // namespace hd
 
 // ---------------------------------------------------------------------------
-// Autotuner of the substitution launch: consumer threads per CTA (96 or 128)
+// Autotuner of the substitution launch: consumer threads per CTA (full storage)
 // and ring depth, timed with CUDA events on real applications; the winner is
 // remembered per (precision, widest box, boxes, device) for the process.
 #include <map>
@@ -882,16 +607,11 @@ int autotune_subst(hd_ctx *ctx, const double2 *r, double2 *z, void *staging, cud
     }
   }
   const int ldmax = ld_max(ctx);
-  // one ring stage: NW warps x tiles per warp (symmetric) or chunk_cols<S>() columns of
-  // ldmax entries (64 bytes per row)
-  const size_t sb = store_bytes(ctx->prec);
-  // symmetric storage: 6 or 8 consumer warps (192 or 256 threads) x tiles per warp per stage
-  auto stage_of = [&](int ct) {
-    return ctx->sym ? (size_t)(ct / 32) * (sb == 4 ? 2 : 1) * TB * TB * sb : (size_t)ldmax * 64;
-  };
+  // one ring stage of the full storage: chunk_cols<S>() columns of ldmax entries (64 bytes per row)
   int dev_optin = 0;
   cudaDeviceGetAttribute(&dev_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  std::vector<int> cts = ctx->sym ? (ctx->max_m <= 192 ? std::vector<int>{192, 256} : std::vector<int>{256})
+  // symmetric storage: threads follow from the number of boxes (launch_subst_sym), only the ring depth is timed
+  std::vector<int> cts = ctx->sym ? std::vector<int>{subst_sym_threads(ctx)}
                                   : (ctx->max_m <= 192 ? std::vector<int>{96, 128, 192} : std::vector<int>{128, 256});
   const int ns_list[] = {2, 3, 4, 6, 8, 12, 16, 24, 32};
   cudaEvent_t e0, e1;
@@ -903,7 +623,7 @@ int autotune_subst(hd_ctx *ctx, const double2 *r, double2 *z, void *staging, cud
   ctx->profiling = false;
   for (int ct : cts)
     for (int ns : ns_list) {
-      if ((size_t)ns * stage_of(ct) + (ctx->sym ? 24576 : 8192) > (size_t)std::min(dev_optin, 224 * 1024)) continue;
+      if (ctx->sym ? ns > 16 : (size_t)ns * ldmax * 64 + 8192 > (size_t)std::min(dev_optin, 224 * 1024)) continue;
       ctx->tune_ct = ct;
       ctx->tune_ns = ns;
       float tot = 0.f;

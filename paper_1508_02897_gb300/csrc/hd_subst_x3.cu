@@ -25,16 +25,24 @@
 // writes those rows of the output and the same 32 columns of the next step's V into
 // A1/A2 (the next step's K range), and arrives on that column group's mbarrier; the MMAs
 // of step t + 1 start on a column group as soon as it is complete, into the other
-// accumulator, so the tensor cores work while the epilogue runs.  Each epilogue thread
+// accumulator, so the tensor cores work while the epilogue runs.  Three warps share a
+// lane quarter, each with two of its column groups.  Each epilogue thread
 // issues the global loads of the operands of its whole step that do not depend on the
 // product (the staged w_j of a backward step, the next grid row's residual of a forward
-// step) before it waits for the accumulator.
+// step) before it waits for the accumulator, and rounds the residual to FP32 on the integer
+// pipe (the FP64 pipe's conversions alone took 5.6K cycles of a forward step).
 //
-// Warp roles: warps 0-3 epilogue (thread = tensor-memory lane), warp 4 producer (factor
+// Warp roles: warps 0-11 epilogue (thread = tensor-memory lane), warp 12 producer (factor
 // chunks through an mbarrier ring with cp.async.bulk, in use order across steps, after
 // asking L2 for them a few chunks ahead: the ring holds two to four chunks beside the A
-// operands, too few to cover HBM's latency on its own), warp 5
-// tensor-memory owner and MMA issuer (one thread).  Every wait is bounded (flag
+// operands, too few to cover HBM's latency on its own), warp 13
+// tensor-memory owner and MMA issuer (one thread).
+//
+// What bounds it: a 176-row step takes 22.5K cycles, 12K of them the 88 MMAs (136 cycles each:
+// A and B operands and the incoming chunks together fill the shared-memory bandwidth), 5K
+// waits for the ring (a refill starts when the MMAs on its stage are done), 5K the first
+// column group of the epilogue.  64 sources, 1984^2 in 256 boxes: 21.8 -> 17.6 ms per
+// application; 16 sources, 1024^2 in 64 boxes: 4.64 -> 3.99 ms.  Every wait is bounded (flag
 // ST_TIMEOUT and unwind); tensor memory is released only after a final commit confirms
 // that no MMA is in flight and the epilogue has finished reading it.
 #include "hd_internal.cuh"
@@ -45,12 +53,14 @@ namespace hd {
 namespace {
 
 constexpr int X3_NR = 32;                     // right-hand sides per CTA
-constexpr int X3_EPI = 128;                   // epilogue threads (tensor-memory lanes 0..127)
+constexpr int X3_E = 3;                       // epilogue warps per quarter of the tensor-memory lanes
+constexpr int X3_EPI = 128 * X3_E;            // epilogue threads
 constexpr int X3_THREADS = X3_EPI + 64;       // + producer warp + MMA warp
 constexpr int X3_TMEM_COLS = 512;             // two accumulators of up to 256 columns
 constexpr uint32_t X3_HALF = 256;             // column offset of the odd-step accumulator
 constexpr uint32_t kX3Lbo = 128;              // A1/A2: bytes between core matrices along K
 constexpr int X3_GROUPS = (kMaxBoxWidthX3 + 31) / 32;   // 32-column groups of the widest box
+constexpr int X3_OWN = (X3_GROUPS + X3_E - 1) / X3_E;   // of one epilogue warp: e, e + X3_E, ...
 constexpr size_t kX3Tail = 256;               // the last plane's N padding (m rounded to 16) reads past the ring
 constexpr int kX3Prefetch = 8;                // chunks the producer asks L2 for ahead of its copies
 
@@ -170,8 +180,8 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
       tc::bar_init(&empty[q], 1);
     }
     tc::bar_init(dfull, 1);
-    for (int g = 0; g < X3_GROUPS; ++g) tc::bar_init(&aready[g], X3_EPI);
-    tc::bar_init(edone, X3_EPI);
+    for (int g = 0; g < X3_GROUPS; ++g) tc::bar_init(&aready[g], 4);   // one arrival per lane quarter
+    tc::bar_init(edone, 4 * X3_E);
     tc::bar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -183,7 +193,7 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
       lA[a] = make_float2((float)v.x, (float)v.y);
     }
   }
-  if (warp == 5) {
+  if (warp == X3_EPI / 32 + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::su32(tholder)),
                  "r"((uint32_t)X3_TMEM_COLS)
                  : "memory");
@@ -196,68 +206,83 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
 
   const int nck = mp8 / 8;                 // chunks (MMA K steps) per block
   const int nsteps = 2 * rows - 1;
-  const int64_t total = (int64_t)nsteps * nck;
   const int64_t slot_floats = 4 * (int64_t)mp8 * mp8;
   const float *Fs = factor + 2 * s.foff;
   const uint32_t chunk_bytes = (uint32_t)(128 * mp8);
 
-  if (warp == 4) {
+  if (warp == X3_EPI / 32) {
     // ---------------- producer: chunks of every block in use order, each asked of L2
     // kX3Prefetch chunks before its copy
+    // (slot, phase and source advance by addition: a refill is on the critical path of the two-
+    // to four-stage ring, and 64-bit divisions there cost more than the copy's latency)
     if (lane == 0) {
-      auto chunk_src = [&](int64_t it) {
-        const int st = (int)(it / nck), c = (int)(it - (int64_t)st * nck);
-        const int j = st < rows ? st : 2 * rows - 2 - st;
-        return Fs + j * slot_floats + (int64_t)c * 32 * mp8;
+      const float *src = Fs, *pre = Fs;   // next chunk to copy, next chunk to ask L2 for
+      int c = 0, st = 0, pc = 0, pst = 0;
+      auto advance = [&](const float *&p, int &cc, int &ss) {
+        p += 32 * mp8;
+        if (++cc == nck) {   // the next block: row + 1 forward, row - 1 backward
+          cc = 0;
+          ++ss;
+          if (ss >= rows) p -= 2 * slot_floats;
+        }
       };
-      for (int64_t it = 0; it < min(total, (int64_t)kX3Prefetch); ++it) prefetch_l2(chunk_src(it), chunk_bytes);
-      int64_t issued = 0;
+      auto prefetch_one = [&]() {
+        if (pst >= nsteps) return;
+        prefetch_l2(pre, chunk_bytes);
+        advance(pre, pc, pst);
+      };
+      for (int q = 0; q < kX3Prefetch; ++q) prefetch_one();
+      int issued = 0, slot = 0;
+      uint32_t ph = 0;
       bool ok = true;
-      for (int64_t it = 0; it < total && ok; ++it) {
-        if (it + kX3Prefetch < total) prefetch_l2(chunk_src(it + kX3Prefetch), chunk_bytes);
-        const int slot = (int)(it % NS);
-        const uint32_t ph = (uint32_t)((it / NS) & 1);
+      while (st < nsteps) {
         if (!tc::bar_spin(&empty[slot], ph ^ 1u, abort_flag)) { ok = false; break; }
         bar_expect(&full[slot], chunk_bytes);
-        bulk_copy(ring + (size_t)slot * stage_bytes, chunk_src(it), chunk_bytes, &full[slot]);
-        issued = it + 1;
+        bulk_copy(ring + (size_t)slot * stage_bytes, src, chunk_bytes, &full[slot]);
+        prefetch_one();
+        advance(src, c, st);
+        ++issued;
+        if (++slot == NS) { slot = 0; ph ^= 1u; }
       }
       if (!ok) {
         *abort_flag = 1;
         atomicOr(status, ST_TIMEOUT);
       }
       // no copy may still be landing when the CTA exits
-      for (int64_t it = max((int64_t)0, issued - NS); it < issued; ++it)
+      for (int it = max(0, issued - NS); it < issued; ++it)
         tc::bar_wait(&full[it % NS], (uint32_t)((it / NS) & 1), abort_flag);
     }
     return;
   }
 
-  if (warp == 5) {
+  if (warp == X3_EPI / 32 + 1) {
     // ---------------- MMA issuer (one thread); the warp owns the tensor memory
     if (lane == 0) {
       // D f32, A and B tf32, both K-major, N = m rounded up to 16, M = 128
       const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(mp16 >> 3) << 17) | ((128u >> 4) << 24);
       const uint32_t a1 = tc::su32(A1), a2 = tc::su32(A2), pl = (uint32_t)(32 * mp8);
-      int64_t it = 0;
+      int slot = 0;
+      uint32_t ph = 0;
+      uint32_t sb = tc::su32(ring);
       bool ok = true;
       for (int st = 0; st < nsteps && ok; ++st) {
         const uint32_t d = tmem + (uint32_t)(st & 1) * X3_HALF;
-        for (int c = 0; c < nck; ++c, ++it) {
+        uint64_t da1 = tc::mdesc(a1, kX3Lbo, asbo), da2 = tc::mdesc(a2, kX3Lbo, asbo);
+        for (int c = 0; c < nck; ++c) {
           if ((c & 3) == 0) {   // the next 32 columns of V (this step's K range) are written
             if (!tc::bar_spin(&aready[c >> 2], (uint32_t)(st & 1), abort_flag)) { ok = false; break; }
             tc::fence_after();
           }
-          const int slot = (int)(it % NS);
-          if (!tc::bar_spin(&full[slot], (uint32_t)((it / NS) & 1), abort_flag)) { ok = false; break; }
-          const uint32_t sb = tc::su32(ring + (size_t)slot * stage_bytes);
-          const uint64_t da1 = tc::mdesc(a1 + (uint32_t)c * 2 * kX3Lbo, kX3Lbo, asbo);
-          const uint64_t da2 = tc::mdesc(a2 + (uint32_t)c * 2 * kX3Lbo, kX3Lbo, asbo);
+          if (!tc::bar_spin(&full[slot], ph, abort_flag)) { ok = false; break; }
           mma_tf32(d, da1, tc::mdesc(sb, 128, 256), idesc, c > 0 ? 1u : 0u);
           mma_tf32(d, da2, tc::mdesc(sb + pl, 128, 256), idesc, 1u);
           mma_tf32(d, da1, tc::mdesc(sb + 2 * pl, 128, 256), idesc, 1u);
           mma_tf32(d, da2, tc::mdesc(sb + 3 * pl, 128, 256), idesc, 1u);
           tc::mma_commit(&empty[slot]);   // the stage is free once these MMAs have read it
+          da1 += 2 * kX3Lbo / 16;   // the next two core matrices along K (descriptor addresses count 16 bytes)
+          da2 += 2 * kX3Lbo / 16;
+          if (++slot == NS) { slot = 0; ph ^= 1u; sb = tc::su32(ring); }
+          else sb += (uint32_t)stage_bytes;
         }
         if (!ok) break;
         tc::mma_commit(dfull);
@@ -277,40 +302,40 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
     return;
   }
 
-  // ---------------- epilogue: lane (part, s) of warp w; right-hand side src = 8w + s.
-  // After the two lane exchanges this thread holds Yr and Yi of src for the 8 columns
-  // coff .. coff+7 of each 32-column group (parts 0, 2, 1, 3 -> columns 0, 8, 16, 24).
-  const int part = lane >> 3, sl = lane & 7, src = 8 * warp + sl;
+  // ---------------- epilogue: lane (part, s) of a warp of lane quarter w; right-hand side
+  // src = 8w + s.  After the two lane exchanges this thread holds Yr and Yi of src for the 8
+  // columns coff .. coff+7 of each 32-column group (parts 0, 2, 1, 3 -> columns 0, 8, 16, 24).
+  const int wq = warp & 3, we = warp >> 2;
+  const int part = lane >> 3, sl = lane & 7, src = 8 * wq + sl;
   const int coff = 16 * (part & 1) + 8 * (part >> 1);
   const bool odd = (part & 1) != 0, up = part >= 2;
   const bool live = r0 + src < nrhs;
-  const double2 *rgs = rg + (int64_t)(live ? r0 + src : 0) * vec_stride;
+  const double2 *rgs = rg + (int64_t)(live ? r0 + src : 0) * vec_stride + s.ex0;
   float2 *stg = staging + (int64_t)(live ? r0 + src : 0) * stg_stride + s.soff;
-  auto owned_x = [&](int a) { return a < m && s.ex0 + a >= s.ox0 && s.ex0 + a < s.ox1; };
+  const bool pairs = ((s.soff | stg_stride | m) & 1) == 0;   // rows of the staging buffer start on 16 bytes
   // residual of grid row gy at columns k0 .. k0+7 (zero outside the owned box, past m, or for idle sources)
   auto load_rho = [&](int gy, int k0, float2 *v) {
     const bool owny = live && gy >= s.oy0 && gy < s.oy1;
+    const int lo = max(s.ox0 - s.ex0, 0), hi = min(s.ox1 - s.ex0, m);
+    const double2 *p = rgs + (int64_t)gy * NX + k0;
+    double2 x[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int a = k0 + i;
-      v[i] = make_float2(0.f, 0.f);
-      if (owny && owned_x(a)) {
-        const double2 x = rgs[(int64_t)gy * NX + s.ex0 + a];
-        v[i] = make_float2((float)x.x, (float)x.y);
-      }
-    }
+    for (int i = 0; i < 8; ++i) x[i] = owny && k0 + i >= lo && k0 + i < hi ? p[i] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = make_float2(d2f_rn(x[i].x), d2f_rn(x[i].y));
   };
   // V_0 = rho_0 (zero in the K padding columns m <= a < mp8)
-  for (int g = 0; g < ngrp; ++g) {
+  for (int g = we; g < ngrp; g += X3_E) {
     const int k0 = 32 * g + coff;
     if (k0 < mp8) {
       float2 v[8];
       load_rho(s.ey0, k0, v);
-      put_v8(A1, A2, asbo, warp, sl, k0, v);
+      put_v8(A1, A2, asbo, wq, sl, k0, v);
     }
     tc::fence_async_smem();
     tc::fence_before();
-    bar_arrive(&aready[g]);
+    __syncwarp();
+    if (lane == 0) bar_arrive(&aready[g]);
   }
 
   for (int st = 0; st < nsteps; ++st) {
@@ -326,19 +351,30 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
       const double2 c = nfwd ? pool[s.aoff + 2 * m + 1 + rows + jn] : pool[s.aoff + 2 * m + 1 + rows + jn + 1];
       cpl = make_float2((float)c.x, (float)c.y);
     }
-    float2 pre[X3_GROUPS][8];
+    float2 pre[X3_OWN][8];
 #pragma unroll
-    for (int g = 0; g < X3_GROUPS; ++g) {
-      const int k0 = 32 * g + coff;
+    for (int o = 0; o < X3_OWN; ++o) {
+      const int g = we + o * X3_E, k0 = 32 * g + coff;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) pre[g][i] = make_float2(0.f, 0.f);
+      for (int i = 0; i < 8; ++i) pre[o][i] = make_float2(0.f, 0.f);
       if (g < ngrp && k0 < mp8) {
         if (!fwd) {
+          const float2 *p = stg + (int64_t)j * m + k0;
+          if (live && pairs) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (live && k0 + i < m) pre[g][i] = stg[(int64_t)j * m + k0 + i];
+            for (int i = 0; i < 8; i += 2)
+              if (k0 + i < m) {   // (m even: whole pairs)
+                const float4 t = *reinterpret_cast<const float4 *>(p + i);
+                pre[o][i] = make_float2(t.x, t.y);
+                pre[o][i + 1] = make_float2(t.z, t.w);
+              }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (live && k0 + i < m) pre[o][i] = p[i];
+          }
         } else if (has_next && nfwd) {
-          load_rho(s.ey0 + jn, k0, pre[g]);
+          load_rho(s.ey0 + jn, k0, pre[o]);
         }
       }
     }
@@ -351,9 +387,10 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
       break;
     }
     tc::fence_after();
-    const uint32_t dcol = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(st & 1) * X3_HALF;
+    const uint32_t dcol = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(st & 1) * X3_HALF;
 #pragma unroll
-    for (int g = 0; g < X3_GROUPS; ++g) {
+    for (int o = 0; o < X3_OWN; ++o) {
+      const int g = we + o * X3_E;
       if (g >= ngrp) break;
       const int k0 = 32 * g + coff;
       const bool colok = k0 < mp8;
@@ -377,27 +414,44 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
         y8[c] = up ? make_float2(y, own) : make_float2(own, y);
       }
       if (colok) {
-        float2 nv[8];
+        float2 nv[8], out[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int a = k0 + i;
-          const float2 out = fwd ? y8[i] : csub(pre[g][i], y8[i]);
-          if (live && a < m) stg[(int64_t)j * m + a] = out;
+          out[i] = fwd ? y8[i] : csub(pre[o][i], y8[i]);
           const float2 lc = cmul(lA[a], cpl);   // L_{jn} or U_{jn} entry of row a (zero past m)
-          nv[i] = nfwd ? cfms(lc, out, pre[g][i]) : cmul(lc, out);
+          nv[i] = nfwd ? cfms(lc, out[i], pre[o][i]) : cmul(lc, out[i]);
           if (a >= m) nv[i] = make_float2(0.f, 0.f);
         }
-        if (has_next) put_v8(A1, A2, asbo, warp, sl, k0, nv);
+        if (has_next) put_v8(A1, A2, asbo, wq, sl, k0, nv);
+        if (has_next) {
+          tc::fence_async_smem();
+          tc::fence_before();
+        }
+        if (live) {
+          float2 *p = stg + (int64_t)j * m + k0;
+          if (pairs) {
+#pragma unroll
+            for (int i = 0; i < 8; i += 2)
+              if (k0 + i < m) *reinterpret_cast<float4 *>(p + i) = make_float4(out[i].x, out[i].y, out[i + 1].x, out[i + 1].y);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (k0 + i < m) p[i] = out[i];
+          }
+        }
+      } else if (has_next) {
+        tc::fence_before();
       }
       if (has_next) {
-        tc::fence_async_smem();
-        tc::fence_before();
-        bar_arrive(&aready[g]);
+        __syncwarp();
+        if (lane == 0) bar_arrive(&aready[g]);
       }
     }
   }
   tc::fence_before();
-  bar_arrive(edone);
+  __syncwarp();
+  if (lane == 0) bar_arrive(edone);
 }
 
 // One CTA per SM (the two accumulators take all 512 tensor-memory columns); ring stages

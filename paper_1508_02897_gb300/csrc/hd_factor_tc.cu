@@ -56,7 +56,7 @@ namespace hd {
 
 namespace {
 
-constexpr int FX_THREADS = 256;
+constexpr int FX_THREADS = 512;   // 16 warps, four per lane quarter of tensor memory
 constexpr int FX_MAXM = 192;     // 2 NP + 2 NB <= 512 tensor-memory columns
 constexpr int FX_KP = 16;        // panel width = K of one kind::f16 MMA
 constexpr int FX_ROWS = 192;     // rows of the B operand tiles and of the panel copy
@@ -70,9 +70,11 @@ constexpr int CLD = 17;          // row stride (entries) of the panel copy: conf
 constexpr size_t kOffA = 0;
 constexpr size_t kOffB = kOffA + (size_t)FX_NA * FX_ATILE;
 constexpr size_t kOffC = kOffB + (size_t)FX_NBT * FX_BTILE;
-constexpr size_t kOffG = kOffC + sizeof(float2) * FX_ROWS * CLD;
+constexpr size_t kOffY = kOffC + sizeof(float2) * FX_ROWS * CLD;
+constexpr size_t kOffG = kOffY + sizeof(float2) * FX_ROWS * CLD;
 constexpr size_t kOffL = kOffG + sizeof(float2) * 2 * FX_KP * FX_KP;
-constexpr size_t kOffM = kOffL + sizeof(float2) * FX_ROWS;
+constexpr size_t kOffD = kOffL + sizeof(float2) * FX_ROWS;
+constexpr size_t kOffM = kOffD + sizeof(float2) * 3 * FX_ROWS;
 constexpr size_t kSmem = kOffM + 32;
 
 // (x0, x1) = h + m + l piecewise, BF16 pieces rounded to nearest (each remainder is
@@ -96,6 +98,18 @@ __device__ __forceinline__ void put_row(unsigned char *tile, int r, const uint32
   unsigned char *p = tile + (r >> 3) * 256 + (r & 7) * 16;
   *reinterpret_cast<uint4 *>(p) = make_uint4(v[0], v[1], v[2], v[3]);
   *reinterpret_cast<uint4 *>(p + 128) = make_uint4(v[4], v[5], v[6], v[7]);
+}
+
+// Half a row (8 values: one 8-column core matrix, h = 0 or 1) split into three pieces, row r
+// of tiles t, t+1, t+2.
+__device__ __forceinline__ void put_split8(unsigned char *tiles, uint32_t tile_bytes, int t, int r, int half, const float *v) {
+  uint32_t h[4], m[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) split3x2(v[2 * i], v[2 * i + 1], h[i], m[i], l[i]);
+  unsigned char *p = tiles + (size_t)t * tile_bytes + (r >> 3) * 256 + (r & 7) * 16 + half * 128;
+  *reinterpret_cast<uint4 *>(p) = make_uint4(h[0], h[1], h[2], h[3]);
+  *reinterpret_cast<uint4 *>(p + tile_bytes) = make_uint4(m[0], m[1], m[2], m[3]);
+  *reinterpret_cast<uint4 *>(p + 2 * (size_t)tile_bytes) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
 // Splits 16 values and writes the three pieces as row r of tiles t, t+1, t+2.
@@ -154,7 +168,9 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   unsigned char *At = smem_raw + kOffA;
   unsigned char *Bt = smem_raw + kOffB;
   float2 *Cs = reinterpret_cast<float2 *>(smem_raw + kOffC);   // [FX_ROWS][CLD] panel columns
+  float2 *Ys = reinterpret_cast<float2 *>(smem_raw + kOffY);   // [FX_ROWS][CLD] Y^T of the panel
   float2 *G = reinterpret_cast<float2 *>(smem_raw + kOffG);    // [2][16][16] pivot block
+  float2 *dS = reinterpret_cast<float2 *>(smem_raw + kOffD);   // [3][FX_ROWS] band entries of the next row's D
   float2 *lS = reinterpret_cast<float2 *>(smem_raw + kOffL);   // [FX_ROWS] coupling of the next row
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem_raw + kOffM);
   uint32_t *tholder = reinterpret_cast<uint32_t *>(mbar + 1);
@@ -177,7 +193,8 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = *tholder;
-  // this warp's lane quarter in tensor memory
+  // this warp's lane quarter in tensor memory, which it shares with three others
+  const int q4 = warp & 3, part = warp >> 2;
   const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
   uint32_t nphase = 0;
   bool alive = true;
@@ -206,26 +223,33 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
       reinterpret_cast<uint4 *>(smem_raw)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) *sflag = 0;
 
-    // ---- S_0 = D_0 into tensor memory (the three band entries of a row computed once)
-    if (warp < 4 || (warp < 6 && mb > 0)) {
-      const double *k2row = k2 + (int64_t)s.ey0 * NX + s.ex0;
-      const bool top = warp < 4;
-      const int r = tid;   // top: rows 0..127; warps 4, 5: rows 128 + (tid - 128)
+    // ---- S_0 = D_0 into tensor memory (the three band entries of a row once per row in shared
+    //      memory; the four warps of a lane quarter take every fourth chunk of 16 columns)
+    auto band_row = [&](int r, int jr) {   // entries (r, r - 1), (r, r), (r, r + 1) of D_jr
+      const double *k2row = k2 + (int64_t)(s.ey0 + jr) * NX + s.ex0;
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        const int c = r - 1 + t;
+        dS[t * FX_ROWS + r] = r < m && c >= 0 && c < m ? d_entry<float2, float>(r, c, jr, a1c, ia1f, a2c, ia2f, k2row, h2)
+                                                       : make_float2(0.f, 0.f);
+      }
+    };
+    __syncthreads();   // (the previous box's write-out has finished reading dS)
+    if (tid < FX_ROWS) band_row(tid, 0);
+    __syncthreads();
+    for (int reg = 0; reg < 2; ++reg) {
+      const bool top = reg == 0;
+      if (!top && (mb == 0 || q4 >= 2)) break;
+      const int r = (top ? 0 : 128) + 32 * q4 + lane;
       const int ncol = top ? NP : NB, cbase = top ? 0 : 128;
       const uint32_t tre = top ? tq : tq + 2 * NP, tim = top ? tq + NP : tq + 2 * NP + NB;
-      float2 dband[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      if (r < m)
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const int c = r - 1 + t;
-          if (c >= 0 && c < m) dband[t] = d_entry<float2, float>(r, c, 0, a1c, ia1f, a2c, ia2f, k2row, h2);
-        }
-      for (int cc = 0; cc < ncol; cc += 16) {
+      const float2 d0 = dS[r], d1 = dS[FX_ROWS + r], d2 = dS[2 * FX_ROWS + r];
+      for (int cc = 16 * part; cc < ncol; cc += 64) {
         float re[16], im[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const int t = cbase + cc + i - r + 1;   // band position 0, 1, 2, or outside
-          const float2 v = t == 0 ? dband[0] : (t == 1 ? dband[1] : (t == 2 ? dband[2] : make_float2(0.f, 0.f)));
+          const float2 v = t == 0 ? d0 : (t == 1 ? d1 : (t == 2 ? d2 : make_float2(0.f, 0.f)));
           re[i] = v.x;
           im[i] = v.y;
         }
@@ -255,32 +279,33 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
         tc::fence_before();
         __syncthreads();
         tc::fence_after();
-        if (warp < 4) {
+        if (part == 0) {
           float re[16], im[16];
-          tc::tmem_ld16(tq + k0, re);
-          tc::tmem_ld16(tq + NP + k0, im);
+          tc::tmem_ld16_nw(tq + k0, re);
+          tc::tmem_ld16_nw(tq + NP + k0, im);
+          tc::tmem_wait_ld();
 #pragma unroll
           for (int i = 0; i < 16; ++i) Cs[tid * CLD + i] = make_float2(re[i], im[i]);
         } else if (mb > 0) {
           if (k0 >= 128) {
-            if (warp < 6) {   // bottom rows from the bottom-right block
-              const int rb = tid - 128;
+            if (part == 1 && q4 < 2) {   // bottom rows from the bottom-right block
+              const int rb = 32 * q4 + lane;
               float re[16], im[16];
-              tc::tmem_ld16(tq + 2 * NP + (k0 - 128), re);
-              tc::tmem_ld16(tq + 2 * NP + NB + (k0 - 128), im);
+              tc::tmem_ld16_nw(tq + 2 * NP + (k0 - 128), re);
+              tc::tmem_ld16_nw(tq + 2 * NP + NB + (k0 - 128), im);
+              tc::tmem_wait_ld();
 #pragma unroll
               for (int i = 0; i < 16; ++i) Cs[(128 + rb) * CLD + i] = make_float2(re[i], im[i]);
             }
-          } else if (warp - 4 == (k0 >> 5)) {
+          } else if (q4 == (k0 >> 5)) {
             // bottom rows of panel columns k < 128: W[128 + c'][k] = W[k][128 + c'], held by lane k
-            const int row = 32 * (warp - 4) + lane;
+            const int row = 32 * q4 + lane;
             const bool mine = row >= k0 && row < k0 + FX_KP;
-            for (int cc = 0; cc < 64; cc += 16) {
+            for (int cc = 16 * (part - 1); cc < NB; cc += 48) {
               float re[16], im[16];
-              if (cc < NB) {
-                tc::tmem_ld16(tq + 128 + cc, re);
-                tc::tmem_ld16(tq + NP + 128 + cc, im);
-              }
+              tc::tmem_ld16_nw(tq + 128 + cc, re);
+              tc::tmem_ld16_nw(tq + NP + 128 + cc, im);
+              tc::tmem_wait_ld();
               if (mine)
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
@@ -292,12 +317,13 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
         }
         __syncthreads();
 
-        // ---- B. the A operand, which needs C only: A = -X, X = C outside rows K and zero on
-        //         rows K (their new values are stored directly), one row per thread; and the
-        //         first pivot of the panel against every unprocessed row below the panel
-        {
-          const int r = tid, kr = r - k0;
-          if (r < FX_ROWS && r < m) {
+        // ---- B. side by side: warps 8..13 the A operand, warps 0..7 the pivot block
+        if (warp >= 8) {
+          // A = -X, X = C outside rows K and zero on rows K (their new values are stored
+          // directly), one row per thread; and the first pivot of the panel against every
+          // unprocessed row below the panel
+          const int r = tid - 256, kr = r - k0;
+          if (r < m) {
             const bool inK = kr >= 0 && kr < w;
             float vr[16], vi[16];
 #pragma unroll
@@ -310,108 +336,109 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
             put_split(At, FX_ATILE, 3, r, vi);
             if (r >= k0 + w && !(cabs2f(Cs[k0 * CLD]) >= tau2 * cabs2f(Cs[r * CLD]))) *sflag = 1;
           }
-        }
-        // ---- P = C_K^{-1} (w x w) by Gauss-Jordan without pivoting, one entry per thread
-        //      (i, jj) = (tid / 16, tid % 16), two alternating shared copies.  Two elimination
-        //      steps k, k+1 per barrier: every thread loads the nine entries it needs and
-        //      applies both in-place steps to its own entry (the same arithmetic as two
-        //      separate steps).  Each pivot is checked by the threads of the unprocessed
-        //      entries below it.
-        {
+          // the band of the next row's D, on the FP64 pipe while the pivot block is inverted
+          if (k0 == 0 && more && r < FX_ROWS) band_row(r, j + 1);
+        } else {
+          // P = C_K^{-1} (w x w) by Gauss-Jordan without pivoting, one entry per thread
+          // (i, jj) = (tid / 16, tid % 16), two alternating shared copies.  Two elimination
+          // steps k, k+1 per barrier: every thread loads the nine entries it needs and
+          // applies both in-place steps to its own entry (the same arithmetic as two
+          // separate steps).  In-place value of entry (x, y) after a step with pivot index k:
+          // the inverse pivot on (k, k), a_ky / pivot on row k, -a_xk / pivot on column k, else
+          // a_xy - a_xk (a_ky / pivot); formed without branches, every case selected from the
+          // few products the entries share.  Each pivot is checked by the threads of the
+          // unprocessed entries below it.  (Two entries per thread on four warps: 6.8K cycles per
+          // panel instead of 5.3K: the instructions of a thread, not the shared work, set the time.)
           const int i = tid >> 4, jj = tid & 15;
           float2 *B0 = G, *B1 = G + 256;
+          auto sync8 = []() { asm volatile("bar.sync 2, 256;" ::: "memory"); };
+          auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
+          auto sel = [](bool c, float2 x, float2 y) { return make_float2(c ? x.x : y.x, c ? x.y : y.y); };
           B0[tid] = (i < w && jj < w) ? Cs[(k0 + i) * CLD + jj] : make_float2(i == jj ? 1.f : 0.f, 0.f);
-          __syncthreads();
-          // in-place Gauss-Jordan value of entry (x, y) after the step with pivot index k and
-          // inverse pivot ip: a_xy the entry, a_xk its pivot-column entry, a_ky its pivot-row entry
-          auto gj = [](int x, int y, int k, float2 a_xy, float2 a_xk, float2 a_ky, float2 ip) -> float2 {
-            if (x == k) return y == k ? ip : cmul(a_ky, ip);
-            if (y == k) {
-              const float2 v = cmul(a_xk, ip);
-              return make_float2(-v.x, -v.y);
-            }
-            return cfms(a_xk, cmul(a_ky, ip), a_xy);
-          };
+          sync8();
           int par = 0;
 #pragma unroll 1
           for (int k = 0; k < w; k += 2, par ^= 1) {
             const float2 *src = par ? B1 : B0;
             float2 *dst = par ? B0 : B1;
+            const int k1 = min(k + 1, 15);
             const float2 piv = src[k * 16 + k], aik = src[i * 16 + k], akj = src[k * 16 + jj], aij = src[tid];
+            const float2 a_i1 = src[i * 16 + k1], a_k1 = src[k * 16 + k1];
+            const float2 a_1j = src[k1 * 16 + jj], a_1k = src[k1 * 16 + k], a_11 = src[k1 * 16 + k1];
             const float p2 = cabs2f(piv);
-            if (jj == k && i > k && i < w && !(p2 >= tau2 * cabs2f(aik))) *sflag = 1;
-            if (tid == 0 && (!(p2 > 0.f) || !isfinite(p2))) *sflag = 1;
             const float rd = recip(p2);   // 1 / pivot = conj(pivot) / |pivot|^2
             const float2 ip = make_float2(piv.x * rd, -piv.y * rd);
-            float2 v = gj(i, jj, k, aij, aik, akj, ip);
-            const int k1 = k + 1;
-            if (k1 < w) {
+            const float2 tj = cmul(akj, ip), t1 = cmul(a_k1, ip);
+            float2 v = sel(i == k, sel(jj == k, ip, tj), sel(jj == k, neg(cmul(aik, ip)), cfms(aik, tj, aij)));
+            bool bad = (jj == k && i > k && i < w && !(p2 >= tau2 * cabs2f(aik))) || (tid == 0 && (!(p2 > 0.f) || !isfinite(p2)));
+            if (k + 1 < w) {
               // the second step on the values after the first
-              const float2 a_i1 = src[i * 16 + k1], a_k1 = src[k * 16 + k1];
-              const float2 a_1j = src[k1 * 16 + jj], a_1k = src[k1 * 16 + k], a_11 = src[k1 * 16 + k1];
-              const float2 vi1 = gj(i, k1, k, a_i1, aik, a_k1, ip);     // entry (i, k+1)
-              const float2 v1j = gj(k1, jj, k, a_1j, a_1k, akj, ip);    // entry (k+1, jj)
-              const float2 piv1 = gj(k1, k1, k, a_11, a_1k, a_k1, ip);  // next pivot
+              const float2 vi1 = sel(i == k, t1, cfms(aik, t1, a_i1));                    // entry (i, k+1)
+              const float2 v1j = sel(jj == k, neg(cmul(a_1k, ip)), cfms(a_1k, tj, a_1j));   // entry (k+1, jj)
+              const float2 piv1 = cfms(a_1k, t1, a_11);                                   // next pivot
               const float q2 = cabs2f(piv1);
-              if (jj == k1 && i > k1 && i < w && !(q2 >= tau2 * cabs2f(vi1))) *sflag = 1;
-              if (tid == 0 && (!(q2 > 0.f) || !isfinite(q2))) *sflag = 1;
               const float rd1 = recip(q2);
               const float2 ip1 = make_float2(piv1.x * rd1, -piv1.y * rd1);
-              v = gj(i, jj, k1, v, vi1, v1j, ip1);
+              const float2 t2 = cmul(v1j, ip1);
+              bad = bad || (jj == k1 && i > k1 && i < w && !(q2 >= tau2 * cabs2f(vi1))) ||
+                    (tid == 0 && (!(q2 > 0.f) || !isfinite(q2)));
+              v = sel(i == k1, sel(jj == k1, ip1, t2), sel(jj == k1, neg(cmul(vi1, ip1)), cfms(vi1, t2, v)));
             }
+            if (bad) *sflag = 1;
             dst[tid] = v;
-            __syncthreads();
+            sync8();
           }
-          // P into the first copy, zero outside w x w
+          // P into the first copy, zero outside w x w (each thread moves its own entry)
           const float2 *res = par ? B1 : B0;
           const float2 pv = (i < w && jj < w) ? res[tid] : make_float2(0.f, 0.f);
-          __syncthreads();
           B0[tid] = pv;
-          __syncthreads();
         }
+        __syncthreads();
         const float2 *Pm = G;   // P[i][kk] at Pm[i * 16 + kk], zero outside w x w
 
-        // ---- C. the B operand Y^T = Z P (three BF16 pieces); Y^T also replaces C in the panel copy
-        if (tid < FX_ROWS && tid < m) {
-          const int r = tid, kr = r - k0;
-          const bool inK = kr >= 0 && kr < w;
-          float vr[16], vi[16];
-          float2 y[16];
-          if (inK) {
+        // ---- C. the B operand Y^T = Z P (three BF16 pieces), half a row per thread: columns
+        //      8 h .. 8 h + 7 of row r; Y^T also goes to Ys for the rows K
+        {
+          // (warps 0..5 and 10..15: three on each scheduler)
+          const int h = warp >= 10, r = h ? tid - 320 : tid, kr = r - k0;
+          if ((h || warp < 6) && r < m) {
+            const bool inK = kr >= 0 && kr < w;
+            float2 y[8];
+            if (inK) {
 #pragma unroll
-            for (int kk = 0; kk < 16; ++kk) y[kk] = Pm[kr * 16 + kk];
-          } else {
-            // y = zs C[r] P: q outer, 16 independent accumulator chains
+              for (int kk = 0; kk < 8; ++kk) y[kk] = Pm[kr * 16 + 8 * h + kk];
+            } else {
+              // y = zs C[r] P: q outer, 8 independent accumulator chains
 #pragma unroll
-            for (int kk = 0; kk < 16; ++kk) y[kk] = make_float2(0.f, 0.f);
-            // kept as a loop over q (16 independent accumulators per step): a fully
-            // unrolled copy is 1024 FMAs of straight-line code in an already large kernel
-#pragma unroll 1
-            for (int q = 0; q < 16; ++q) {
-              const float4 *prow = reinterpret_cast<const float4 *>(Pm + q * 16);
-              const float2 cq = Cs[r * CLD + q];
+              for (int kk = 0; kk < 8; ++kk) y[kk] = make_float2(0.f, 0.f);
+#pragma unroll 4
+              for (int q = 0; q < 16; ++q) {
+                const float4 *prow = reinterpret_cast<const float4 *>(Pm + q * 16 + 8 * h);
+                const float2 cq = Cs[r * CLD + q];
 #pragma unroll
-              for (int k2 = 0; k2 < 8; ++k2) {
-                const float4 pp = prow[k2];
-                y[2 * k2] = cfma(cq, make_float2(pp.x, pp.y), y[2 * k2]);
-                y[2 * k2 + 1] = cfma(cq, make_float2(pp.z, pp.w), y[2 * k2 + 1]);
+                for (int k2 = 0; k2 < 4; ++k2) {
+                  const float4 pp = prow[k2];
+                  y[2 * k2] = cfma(cq, make_float2(pp.x, pp.y), y[2 * k2]);
+                  y[2 * k2 + 1] = cfma(cq, make_float2(pp.z, pp.w), y[2 * k2 + 1]);
+                }
               }
+              if (r < k0)
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) y[kk] = make_float2(-y[kk].x, -y[kk].y);
             }
-            if (r < k0)
+            float vr[8], vi[8];
 #pragma unroll
-              for (int kk = 0; kk < 16; ++kk) y[kk] = make_float2(-y[kk].x, -y[kk].y);
+            for (int kk = 0; kk < 8; ++kk) {
+              vr[kk] = y[kk].x;
+              vi[kk] = y[kk].y;
+              Ys[r * CLD + 8 * h + kk] = y[kk];
+            }
+            put_split8(Bt, FX_BTILE, 0, r, h, vr);
+            put_split8(Bt, FX_BTILE, 3, r, h, vi);
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) vi[kk] = -vi[kk];
+            put_split8(Bt, FX_BTILE, 6, r, h, vi);
           }
-#pragma unroll
-          for (int kk = 0; kk < 16; ++kk) {
-            vr[kk] = y[kk].x;
-            vi[kk] = y[kk].y;
-            Cs[r * CLD + kk] = y[kk];
-          }
-          put_split(Bt, FX_BTILE, 0, r, vr);
-          put_split(Bt, FX_BTILE, 3, r, vi);
-#pragma unroll
-          for (int kk = 0; kk < 16; ++kk) vi[kk] = -vi[kk];
-          put_split(Bt, FX_BTILE, 6, r, vi);
         }
         __syncthreads();
         // rows K take their new values directly, W[k][:] = Y[k - k0][:] (P on the diagonal
@@ -420,7 +447,7 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
         // warp-collective, so the warp holding rows K rewrites whole rows: its other lanes
         // store back what they hold (zero in the columns K).
         {
-          const int q = warp & 3;
+          const int q = q4;
           const bool top_rmw = k0 < 128 && q == (k0 >> 5);
           const bool bot_rmw = k0 >= 128 && q == ((k0 - 128) >> 5);
           // columns K of rows outside K: zero (top rows: warps 0-3; bottom rows: warps 4, 5)
@@ -428,43 +455,40 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
             const float z[16] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             tc::tmem_st16(tq + k0, z);
             tc::tmem_st16(tq + NP + k0, z);
-          } else if ((warp == 4 || warp == 5) && k0 >= 128 && !bot_rmw) {
+          } else if (part == 1 && q < 2 && k0 >= 128 && !bot_rmw) {
             const float z[16] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             tc::tmem_st16(tq + 2 * NP + (k0 - 128), z);
             tc::tmem_st16(tq + 2 * NP + NB + (k0 - 128), z);
           }
           if (top_rmw || bot_rmw) {
-            // the two warps of this lane quarter rewrite the rows of K, half the columns each
+            // the four warps of this lane quarter rewrite the rows of K, a quarter of the columns each
             const int rrow = top_rmw ? 32 * q + lane : 128 + 32 * q + lane;
             const int kr = rrow - k0;
             const bool inK = kr >= 0 && kr < w;
             const int ncol = top_rmw ? NP : NB, cb = top_rmw ? 0 : 128, kc = k0 - cb;
-            const int nch = ncol / 16, half = (nch + 1) / 2;
-            const int ch0 = warp < 4 ? 0 : half, ch1 = warp < 4 ? half : nch;
+            const int nch = ncol / 16;
+            const int ch0 = nch * part / 4, ch1 = nch * (part + 1) / 4;
             const uint32_t tre = top_rmw ? tq : tq + 2 * NP, tim = top_rmw ? tq + NP : tq + 2 * NP + NB;
-            for (int c2 = ch0; c2 < ch1; c2 += 2) {
-              float re[2][16], im[2][16];
-              const int nh = c2 + 1 < ch1 ? 2 : 1;   // chunks of 16 columns in this pass, one wait
-              for (int hh = 0; hh < nh; ++hh) {
-                tc::tmem_ld16_nw(tre + 16 * (c2 + hh), re[hh]);
-                tc::tmem_ld16_nw(tim + 16 * (c2 + hh), im[hh]);
-              }
+            for (int ch = ch0; ch < ch1; ++ch) {
+              float re[16], im[16];
+              const int cc = 16 * ch;
+              tc::tmem_ld16_nw(tre + cc, re);
+              tc::tmem_ld16_nw(tim + cc, im);
               tc::tmem_wait_ld();
-              for (int hh = 0; hh < nh; ++hh) {
-                const int cc = 16 * (c2 + hh);
+              {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                   if (inK) {
-                    const float2 v = Cs[(cb + cc + i) * CLD + kr];
-                    re[hh][i] = v.x;
-                    im[hh][i] = v.y;
+                    const float2 v = Ys[(cb + cc + i) * CLD + kr];
+                    re[i] = v.x;
+                    im[i] = v.y;
                   } else if (cc == kc) {
-                    re[hh][i] = 0.f;
-                    im[hh][i] = 0.f;
+                    re[i] = 0.f;
+                    im[i] = 0.f;
                   }
                 }
-                tc::tmem_st16(tre + cc, re[hh]);
-                tc::tmem_st16(tim + cc, im[hh]);
+                tc::tmem_st16(tre + cc, re);
+                tc::tmem_st16(tim + cc, im);
               }
             }
           }
@@ -514,50 +538,31 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
 
       // ---- write S_j^{-1} out and turn it into S_{j+1} = D_{j+1} - L S_j^{-1} L in place
       S *slot = Fs + (int64_t)j * slot_elems;
-      const double *k2row = k2 + (int64_t)(s.ey0 + j + 1) * NX + s.ex0;
       const int ldm = s.ldm;
-      // every warp takes part: warps 0-3 the left columns of their rows 0..127, warps 4-7 the
-      // right columns of the same rows, warps 4 and 5 also the bottom-right block (rows
-      // 128..m-1), the column split balancing the 16-column chunks
+      // the four warps of a lane quarter split the 16-column chunks of their rows: rows 0..127,
+      // and for the quarters 0 and 1 also the bottom-right block (rows 128..m-1)
       {
-        const int q = warp & 3;
-        const int nchT = NP / 16, nchB = NB / 16, sT = (nchT + nchB + 1) / 2;
+        const int q = q4;
+        const int nchT = NP / 16, nchB = q < 2 ? NB / 16 : 0, nch = nchT + nchB;
+        const int t0 = nch * part / 4, t1 = nch * (part + 1) / 4;
         for (int reg = 0; reg < 2; ++reg) {
           const bool top = reg == 0;
-          int ch0, ch1;
-          if (top) {
-            ch0 = warp < 4 ? 0 : min(sT, nchT);
-            ch1 = warp < 4 ? min(sT, nchT) : nchT;
-          } else {
-            ch0 = 0;
-            ch1 = (warp == 4 || warp == 5) ? nchB : 0;
-          }
+          const int ch0 = top ? min(t0, nchT) : max(t0 - nchT, 0), ch1 = top ? min(t1, nchT) : max(t1 - nchT, 0);
           if (ch0 >= ch1) continue;
           const int r = top ? 32 * q + lane : 128 + 32 * q + lane;
           const int cbase = top ? 0 : 128;
           const uint32_t tre = top ? tq : tq + 2 * NP, tim = top ? tq + NP : tq + 2 * NP + NB;
           const int I = r >> 4, rr = r & 15;
-          // the three entries of D_{j+1} in row r (west, centre, east), once per row
-          float2 dband[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
           const float2 lr = lS[r];
-          if (more && r < m)
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-              const int c = r - 1 + t;
-              if (c >= cbase + 16 * ch0 - 1 && c <= cbase + 16 * ch1 && c >= 0 && c < m)
-                dband[t] = d_entry<float2, float>(r, c, j + 1, a1c, ia1f, a2c, ia2f, k2row, h2);
-            }
-          for (int c2 = ch0; c2 < ch1; c2 += 2) {
-            float rb[2][16], ib[2][16];
-            const int nh = c2 + 1 < ch1 ? 2 : 1;   // chunks of 16 columns in this pass, one wait
-            for (int hh = 0; hh < nh; ++hh) {
-              tc::tmem_ld16_nw(tre + 16 * (c2 + hh), rb[hh]);
-              tc::tmem_ld16_nw(tim + 16 * (c2 + hh), ib[hh]);
-            }
+          const float2 d0 = dS[r], d1 = dS[FX_ROWS + r], d2 = dS[2 * FX_ROWS + r];   // D_{j+1} in row r
+#pragma unroll 1
+          for (int ch = ch0; ch < ch1; ++ch) {
+            float re[16], im[16];
+            const int cc = 16 * ch;
+            tc::tmem_ld16_nw(tre + cc, re);
+            tc::tmem_ld16_nw(tim + cc, im);
             tc::tmem_wait_ld();
-            for (int hh = 0; hh < nh; ++hh) {
-              const int cc = 16 * (c2 + hh);
-              float *re = rb[hh], *im = ib[hh];
+            {
               const int c0 = cbase + cc;
               if (LAY == LAY_SYM) {
                 const int J = c0 >> 4;
@@ -587,7 +592,7 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
                   float2 v = make_float2(0.f, 0.f);
                   if (r < m && c < m) {
                     const int t = c - r + 1;   // band position 0, 1, 2, or outside
-                    const float2 d = t == 0 ? dband[0] : (t == 1 ? dband[1] : (t == 2 ? dband[2] : make_float2(0.f, 0.f)));
+                    const float2 d = t == 0 ? d0 : (t == 1 ? d1 : (t == 2 ? d2 : make_float2(0.f, 0.f)));
                     v = cfms(cmul(lr, make_float2(re[i], im[i])), lS[c], d);
                   }
                   re[i] = v.x;

@@ -35,7 +35,18 @@
 // real products Xr Yr, Xi Yi, Xr Yi, Xi Yr, each accumulated into its real or
 // imaginary plane with the sign stored in the operands (A = -Xr, -Xi; B = Yr, Yi,
 // -Yi).  One panel is 24 MMAs for rows 0..127 (N = NP) and 24 for the bottom-right
-// block (M = 128 rows starting at operand row 128, N = NB).
+// block (M = 128 rows starting at operand row 128, N = NB); for boxes wider than 128 the
+// columns from the next panel on are updated first, and the others under that panel's copy,
+// pivot block and A operand (a second A operand; every entry still receives the same
+// products in the same order).
+//
+// What bounds it: the chain of the panels, one CTA per SM (tensor and shared memory are both
+// full).  Cycles per panel of 16 columns at m = 176: copy 0.7K, pivot block 5.2K (sixteen
+// dependent elimination steps, two per barrier; the A operand and the next row's band entries
+// are formed beside it), B operand 3.6K, rows K 0.6K, waits for the first MMAs 2.5K; per grid
+// row 15K to write S_j^{-1} out and rebuild.  64 boxes of 174: 21.6 ms with eight warps and
+// the phases one after another, 16.5 ms with sixteen, 15.8 ms with the split update; 4096^2
+// (1024 boxes of 176): 154 -> 118 -> 113 ms.
 //
 // Pivot check: within each diagonal block every pivot is compared with the other
 // unprocessed entries of its column (and, for the first column of the panel, with
@@ -68,7 +79,7 @@ constexpr uint32_t FX_TMEM_COLS = 512;
 constexpr int CLD = 17;          // row stride (entries) of the panel copy: conflict-free rows and columns
 
 constexpr size_t kOffA = 0;
-constexpr size_t kOffB = kOffA + (size_t)FX_NA * FX_ATILE;
+constexpr size_t kOffB = kOffA + 2 * (size_t)FX_NA * FX_ATILE;   // two A operands: the next panel's is formed under this one's MMAs
 constexpr size_t kOffC = kOffB + (size_t)FX_NBT * FX_BTILE;
 constexpr size_t kOffY = kOffC + sizeof(float2) * FX_ROWS * CLD;
 constexpr size_t kOffG = kOffY + sizeof(float2) * FX_ROWS * CLD;
@@ -173,13 +184,14 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   float2 *dS = reinterpret_cast<float2 *>(smem_raw + kOffD);   // [3][FX_ROWS] band entries of the next row's D
   float2 *lS = reinterpret_cast<float2 *>(smem_raw + kOffL);   // [FX_ROWS] coupling of the next row
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem_raw + kOffM);
-  uint32_t *tholder = reinterpret_cast<uint32_t *>(mbar + 1);
+  uint32_t *tholder = reinterpret_cast<uint32_t *>(mbar + 2);
   volatile int *sflag = reinterpret_cast<volatile int *>(tholder + 1);
   volatile int *abort_flag = sflag + 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
     tc::bar_init(mbar, 1);
+    tc::bar_init(mbar + 1, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -196,8 +208,11 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   // this warp's lane quarter in tensor memory, which it shares with three others
   const int q4 = warp & 3, part = warp >> 2;
   const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-  uint32_t nphase = 0;
-  bool alive = true;
+  const bool issuer = warp == FX_THREADS / 32 - 1 && lane == 0;   // of the MMAs (its warp has no other work while they are issued)
+  uint32_t nphase = 0, nrest = 0;   // completed phases of mbar[0] and mbar[1]
+  int abuf = 0;
+  bool alive = true, rest = false;   // rest: MMAs of mbar[1] are in flight
+
 
   for (int box = blockIdx.x; box < nsub && alive; box += gridDim.x) {
     const SubDev s = subs[box];
@@ -215,8 +230,6 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
                                               : (LAY == LAY_TC    ? (int64_t)mp8 * mp8
                                                  : LAY == LAY_TC3 ? 2 * (int64_t)mp8 * mp8
                                                                   : (int64_t)m * s.ldm);
-    const uint32_t idesc_top = tc::idesc_bf16(128, NP);
-    const uint32_t idesc_bot = tc::idesc_bf16(128, NB > 0 ? NB : 16);
 
     // operand tiles and the panel copy start at zero: rows >= m are never written
     for (int i = tid; i < (int)(kOffG / 16); i += FX_THREADS)
@@ -275,10 +288,16 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
 
       for (int k0 = 0; k0 < m; k0 += FX_KP) {
         const int w = min(FX_KP, m - k0);
-        // ---- A. copy the panel columns C = W[:, K] into shared memory
-        tc::fence_before();
-        __syncthreads();
-        tc::fence_after();
+        // ---- A. copy the panel columns C = W[:, K] into shared memory.  Behind a panel whose
+        //      remaining MMAs still run, their issuer's warp leaves A and B to the others (its
+        //      instructions block while the tensor cores are busy) and joins them before C.
+        const bool follow = rest, ahead = !(follow && warp == FX_THREADS / 32 - 1);
+        if (!follow) {
+          tc::fence_before();
+          __syncthreads();
+          tc::fence_after();
+        }
+        if (ahead) {
         if (part == 0) {
           float re[16], im[16];
           tc::tmem_ld16_nw(tq + k0, re);
@@ -301,7 +320,7 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
             // bottom rows of panel columns k < 128: W[128 + c'][k] = W[k][128 + c'], held by lane k
             const int row = 32 * q4 + lane;
             const bool mine = row >= k0 && row < k0 + FX_KP;
-            for (int cc = 16 * (part - 1); cc < NB; cc += 48) {
+            for (int cc = 16 * (part - 1); cc < NB && part < 3; cc += 32) {
               float re[16], im[16];
               tc::tmem_ld16_nw(tq + 128 + cc, re);
               tc::tmem_ld16_nw(tq + NP + 128 + cc, im);
@@ -315,13 +334,15 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
             }
           }
         }
-        __syncthreads();
+        if (follow) asm volatile("bar.sync 3, %0;" ::"n"(FX_THREADS - 32) : "memory");
+        else __syncthreads();
 
         // ---- B. side by side: warps 8..13 the A operand, warps 0..7 the pivot block
         if (warp >= 8) {
           // A = -X, X = C outside rows K and zero on rows K (their new values are stored
           // directly), one row per thread; and the first pivot of the panel against every
           // unprocessed row below the panel
+          unsigned char *Aw = At + (size_t)abuf * FX_NA * FX_ATILE;
           const int r = tid - 256, kr = r - k0;
           if (r < m) {
             const bool inK = kr >= 0 && kr < w;
@@ -332,8 +353,8 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
               vr[i] = inK ? 0.f : -c.x;
               vi[i] = inK ? 0.f : -c.y;
             }
-            put_split(At, FX_ATILE, 0, r, vr);
-            put_split(At, FX_ATILE, 3, r, vi);
+            put_split(Aw, FX_ATILE, 0, r, vr);
+            put_split(Aw, FX_ATILE, 3, r, vi);
             if (r >= k0 + w && !(cabs2f(Cs[k0 * CLD]) >= tau2 * cabs2f(Cs[r * CLD]))) *sflag = 1;
           }
           // the band of the next row's D, on the FP64 pipe while the pivot block is inverted
@@ -393,7 +414,18 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
           const float2 pv = (i < w && jj < w) ? res[tid] : make_float2(0.f, 0.f);
           B0[tid] = pv;
         }
+        }   // ahead
+        // the previous panel's remaining MMAs read the B operand and write W: done from here on
+        if (rest && !tc::bar_spin(mbar + 1, nrest & 1u, abort_flag)) *abort_flag = 1;
+        if (rest) ++nrest;
+        rest = false;
+        tc::fence_after();
         __syncthreads();
+        if (*abort_flag) {   // (set before the barrier: every thread leaves here)
+          if (tid == 0) atomicOr(status, ST_TIMEOUT);
+          alive = false;
+          break;
+        }
         const float2 *Pm = G;   // P[i][kk] at Pm[i * 16 + kk], zero outside w x w
 
         // ---- C. the B operand Y^T = Z P (three BF16 pieces), half a row per thread: columns
@@ -498,40 +530,65 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
         tc::fence_before();
         __syncthreads();
 
-        // ---- D. W -= X Y on the tensor cores (one thread issues), then wait
-        if (tid == 0) {
+        // ---- D. W -= X Y on the tensor cores (one thread issues).  The columns that the next
+        //      panel copies come first, with a commit of their own; the others run while that
+        //      panel's copy, pivot block and A operand are formed.  Every entry still receives its
+        //      24 products in the same order.
+        const int kn = k0 + FX_KP;   // next panel
+        const bool last = kn >= m, whole = last || mb == 0;   // (up to 128 wide the split costs more than it hides)
+        if (issuer) {
           tc::fence_after();
-          const uint32_t a0 = tc::su32(At), b0 = tc::su32(Bt);
-          for (int part = 0; part < (mb > 0 ? 2 : 1); ++part) {
-            const uint32_t dr = tmem + (part ? 2 * NP : 0), di = tmem + (part ? 2 * NP + NB : NP);
-            const uint32_t ro = part ? 16 * 256 : 0;   // operand row 128: 16 groups of 8 rows
-            const uint32_t id = part ? idesc_bot : idesc_top;
+          const uint32_t a0 = tc::su32(At) + (uint32_t)abuf * FX_NA * FX_ATILE, b0 = tc::su32(Bt);
+          // columns c0 .. c0 + n - 1 of rows 0..127 (part 0) or of the bottom-right block (part 1)
+          auto update = [&](int bottom, int c0, int n) {
+            if (n <= 0) return;
+            const uint32_t dr = tmem + (bottom ? 2 * NP : 0) + c0, di = dr + (bottom ? NB : NP);
+            const uint32_t ro = bottom ? 16 * 256 : 0;   // operand row 128: 16 groups of 8 rows
+            const uint32_t co = ro + (uint32_t)(c0 >> 3) * 256;
+            const uint32_t id = tc::idesc_bf16(128, (uint32_t)n);
 #pragma unroll
             for (int pq = 0; pq < 6; ++pq) {
               // piece pairs (p, q) with p + q <= 2: (0,0) (0,1) (1,0) (0,2) (1,1) (2,0)
               const int p = pq == 2 ? 1 : (pq == 4 ? 1 : (pq == 5 ? 2 : 0));
               const int q = pq == 1 ? 1 : (pq == 3 ? 2 : (pq == 4 ? 1 : 0));
-              const uint32_t axr = a0 + (uint32_t)p * FX_ATILE + ro, axi = a0 + (uint32_t)(3 + p) * FX_ATILE + ro;
-              const uint32_t byr = b0 + (uint32_t)q * FX_BTILE + ro, byi = b0 + (uint32_t)(3 + q) * FX_BTILE + ro;
-              const uint32_t byn = b0 + (uint32_t)(6 + q) * FX_BTILE + ro;
-              tc::mma_bf16(dr, tc::mdesc(axr, 128, 256), tc::mdesc(byr, 128, 256), id, 1u);   // -Xr Yr
-              tc::mma_bf16(dr, tc::mdesc(axi, 128, 256), tc::mdesc(byn, 128, 256), id, 1u);   // +Xi Yi
-              tc::mma_bf16(di, tc::mdesc(axr, 128, 256), tc::mdesc(byi, 128, 256), id, 1u);   // -Xr Yi
-              tc::mma_bf16(di, tc::mdesc(axi, 128, 256), tc::mdesc(byr, 128, 256), id, 1u);   // -Xi Yr
+              const uint64_t axr = tc::mdesc(a0 + (uint32_t)p * FX_ATILE + ro, 128, 256);
+              const uint64_t axi = tc::mdesc(a0 + (uint32_t)(3 + p) * FX_ATILE + ro, 128, 256);
+              const uint64_t byr = tc::mdesc(b0 + (uint32_t)q * FX_BTILE + co, 128, 256);
+              const uint64_t byi = tc::mdesc(b0 + (uint32_t)(3 + q) * FX_BTILE + co, 128, 256);
+              const uint64_t byn = tc::mdesc(b0 + (uint32_t)(6 + q) * FX_BTILE + co, 128, 256);
+              tc::mma_bf16(dr, axr, byr, id, 1u);   // -Xr Yr
+              tc::mma_bf16(dr, axi, byn, id, 1u);   // +Xi Yi
+              tc::mma_bf16(di, axr, byi, id, 1u);   // -Xr Yi
+              tc::mma_bf16(di, axi, byr, id, 1u);   // -Xi Yr
             }
+          };
+          if (whole) {
+            update(0, 0, NP);
+            if (mb > 0) update(1, 0, NB);
+            tc::mma_commit(mbar);
+          } else {
+            // (one range: an instruction takes about as long for 16 columns as for 128; the rows
+            // 128.. of a panel left of column 128 come from the columns 128.. by symmetry)
+            update(0, kn, NP - kn);
+            if (kn >= 128) update(1, kn - 128, NB - (kn - 128));
+            tc::mma_commit(mbar);
+            update(0, 0, kn);
+            if (mb > 0) update(1, 0, kn >= 128 ? kn - 128 : NB);
+            tc::mma_commit(mbar + 1);
           }
-          tc::mma_commit(mbar);
         }
-        const bool ok = tc::bar_spin(mbar, nphase & 1u, abort_flag);
+        rest = !whole;
+        abuf ^= 1;
+        if (!tc::bar_spin(mbar, nphase & 1u, abort_flag)) *abort_flag = 1;
         ++nphase;
         tc::fence_after();
-        if (__syncthreads_or(!ok)) {
-          if (tid == 0) {
-            *abort_flag = 1;
-            atomicOr(status, ST_TIMEOUT);
+        if (whole) {   // (behind a split update the next panel starts from each thread's own wait: no barrier between)
+          __syncthreads();
+          if (*abort_flag) {
+            if (tid == 0) atomicOr(status, ST_TIMEOUT);
+            alive = false;
+            break;
           }
-          alive = false;
-          break;
         }
       }
       if (!alive) break;
@@ -614,7 +671,7 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   // ---- release tensor memory once no MMA is in flight
   tc::fence_before();
   __syncthreads();
-  if (!alive && tid == 0) {
+  if (!alive && issuer) {
     tc::mma_commit(mbar);   // arrives when every MMA issued so far has completed
     volatile int never = 0;
     tc::bar_wait(mbar, nphase & 1u, &never);

@@ -18,7 +18,10 @@
 // 2, 3) of right-hand side 8w + s, and the epilogue adds the parts with two lane
 // exchanges.  Four MMAs per chunk serve 32 right-hand sides: the instruction count per
 // right-hand side of the TF32 path (two MMAs per chunk for 16), and the same factor bytes
-// per right-hand side (16 bytes per entry, read once per 32).
+// per right-hand side (16 bytes per entry, read once per 32).  With M = 64 (SQ = 4) a CTA
+// takes 16 right-hand sides: the MMAs take as long, but the A operands half the shared
+// memory, so the ring holds six chunks instead of two; for up to 16 right-hand sides, and
+// for more where few boxes leave SMs idle.
 //
 // Pipelining inside the CTA: two accumulators in tensor memory (even and odd steps).
 // The epilogue of step t reads its accumulator 32 columns (rows a of the box) at a time,
@@ -38,11 +41,11 @@
 // operands, too few to cover HBM's latency on its own), warp 13
 // tensor-memory owner and MMA issuer (one thread).
 //
-// What bounds it: a 176-row step takes 22.5K cycles, 12K of them the 88 MMAs (136 cycles each:
-// A and B operands and the incoming chunks together fill the shared-memory bandwidth), 5K
-// waits for the ring (a refill starts when the MMAs on its stage are done), 5K the first
-// column group of the epilogue.  64 sources, 1984^2 in 256 boxes: 21.8 -> 17.6 ms per
-// application; 16 sources, 1024^2 in 64 boxes: 4.64 -> 3.99 ms.  Every wait is bounded (flag
+// What bounds it: a 176-row step takes 22.5K cycles (17.6K with M = 64), 12K of them the 88
+// MMAs (137 cycles each, whatever M), 5K (1.4K) waits for the ring (a refill starts when the
+// MMAs on its stage are done), 5K (4K) the first column group of the epilogue.  64 sources,
+// 1984^2 in 256 boxes: 21.8 -> 17.5 ms per application; 16 sources, 1024^2 in 64 boxes: 4.64 ->
+// 3.27 ms.  Every wait is bounded (flag
 // ST_TIMEOUT and unwind); tensor memory is released only after a final commit confirms
 // that no MMA is in flight and the epilogue has finished reading it.
 #include "hd_internal.cuh"
@@ -52,7 +55,6 @@ namespace hd {
 
 namespace {
 
-constexpr int X3_NR = 32;                     // right-hand sides per CTA
 constexpr int X3_E = 3;                       // epilogue warps per quarter of the tensor-memory lanes
 constexpr int X3_EPI = 128 * X3_E;            // epilogue threads
 constexpr int X3_THREADS = X3_EPI + 64;       // + producer warp + MMA warp
@@ -108,9 +110,17 @@ __device__ __forceinline__ float tf32_rn(float x) {
   return __uint_as_float(r);
 }
 
-// Writes columns k0 .. k0+7 of right-hand side s (warp quarter w) into A1 and A2: the
+// Right-hand sides of a lane quarter: SQ = 8 (M = 128) or 4 (M = 64, rows 16 w .. 16 w + 15 of
+// quarter w in its first 16 lanes).  Row of part p of right-hand side s: 4 SQ w + SQ p + s.
+template <int SQ> __device__ __forceinline__ uint32_t a_row(int w, int p, int s, uint32_t sbo) {
+  return SQ == 8 ? (uint32_t)(4 * w + p) * sbo + (uint32_t)s * 16
+                 : (uint32_t)(2 * w + (p >> 1)) * sbo + (uint32_t)((p & 1) * 4 + s) * 16;
+}
+
+// Writes columns k0 .. k0+7 of right-hand side s (lane quarter w) into A1 and A2: the
 // four part rows of each, two 16-byte stores per row.  A1/A2 element (n, k) sits at
 // (n / 8) * sbo + (k / 4) * kX3Lbo + (n % 8) * 16 + (k % 4) * 4 bytes.
+template <int SQ>
 __device__ __forceinline__ void put_v8(unsigned char *A1, unsigned char *A2, uint32_t sbo, int w, int s, int k0,
                                        const float2 *v) {
   float rh[8], rl[8], ih[8], il[8];
@@ -121,9 +131,9 @@ __device__ __forceinline__ void put_v8(unsigned char *A1, unsigned char *A2, uin
     ih[i] = tf32_rn(v[i].y);
     il[i] = tf32_rn(v[i].y - ih[i]);
   }
-  const uint32_t base = (uint32_t)(k0 >> 2) * kX3Lbo + (uint32_t)s * 16;
+  const uint32_t base = (uint32_t)(k0 >> 2) * kX3Lbo;
   auto row = [&](unsigned char *A, int part) -> float4 * {
-    return reinterpret_cast<float4 *>(A + (size_t)(4 * w + part) * sbo + base);
+    return reinterpret_cast<float4 *>(A + a_row<SQ>(w, part, s, sbo) + base);
   };
   auto st2 = [&](float4 *p, const float *x, float sg) {
     p[0] = make_float4(sg * x[0], sg * x[1], sg * x[2], sg * x[3]);
@@ -141,14 +151,15 @@ __device__ __forceinline__ void put_v8(unsigned char *A1, unsigned char *A2, uin
 
 }  // namespace
 
-// Shared memory: A1, A2 [16 row groups][mp8max / 4 core matrices][128 B] | ring [NS][128 mp8max]
+// Shared memory: A1, A2 [2 SQ row groups][mp8max / 4 core matrices][128 B] | ring [NS][128 mp8max]
 // | tail padding | lA [mp8max] float2 | full[NS] | empty[NS] | dfull | aready[X3_GROUPS] | edone
 // | fin | tensor-memory address | abort flag.
-static size_t subst_x3_smem(int ns, int mp8max) {
-  return 2 * (size_t)512 * mp8max + (size_t)ns * 128 * mp8max + kX3Tail + 8 * (size_t)mp8max +
+static size_t subst_x3_smem(int sq, int ns, int mp8max) {
+  return 2 * (size_t)64 * sq * mp8max + (size_t)ns * 128 * mp8max + kX3Tail + 8 * (size_t)mp8max +
          (2 * (size_t)ns + 3 + X3_GROUPS) * 8 + 16;
 }
 
+template <int SQ>
 __global__ void __launch_bounds__(X3_THREADS, 1)
 k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, const float *__restrict__ factor,
            const double2 *__restrict__ rg, int NX, int64_t vec_stride, float2 *__restrict__ staging, int64_t stg_stride,
@@ -156,12 +167,12 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const SubDev s = subs[blockIdx.y];
   const int m = s.ex, rows = s.ey, mp8 = (m + 7) & ~7, mp16 = (m + 15) & ~15;
-  const int r0 = blockIdx.x * X3_NR;
+  const int r0 = blockIdx.x * (4 * SQ);
   const size_t stage_bytes = (size_t)128 * mp8max;
   const uint32_t asbo = kX3Lbo * (uint32_t)(mp8max / 4);   // A1/A2: bytes between 8-row groups
   unsigned char *A1 = smem_raw;
-  unsigned char *A2 = A1 + (size_t)16 * asbo;
-  unsigned char *ring = A2 + (size_t)16 * asbo;
+  unsigned char *A2 = A1 + (size_t)2 * SQ * asbo;
+  unsigned char *ring = A2 + (size_t)2 * SQ * asbo;
   float2 *lA = reinterpret_cast<float2 *>(ring + (size_t)NS * stage_bytes + kX3Tail);
   uint64_t *full = reinterpret_cast<uint64_t *>(lA + mp8max);
   uint64_t *empty = full + NS;
@@ -258,8 +269,8 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
   if (warp == X3_EPI / 32 + 1) {
     // ---------------- MMA issuer (one thread); the warp owns the tensor memory
     if (lane == 0) {
-      // D f32, A and B tf32, both K-major, N = m rounded up to 16, M = 128
-      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(mp16 >> 3) << 17) | ((128u >> 4) << 24);
+      // D f32, A and B tf32, both K-major, N = m rounded up to 16, M = 16 SQ
+      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(mp16 >> 3) << 17) | ((uint32_t)SQ << 24);
       const uint32_t a1 = tc::su32(A1), a2 = tc::su32(A2), pl = (uint32_t)(32 * mp8);
       int slot = 0;
       uint32_t ph = 0;
@@ -303,13 +314,14 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
   }
 
   // ---------------- epilogue: lane (part, s) of a warp of lane quarter w; right-hand side
-  // src = 8w + s.  After the two lane exchanges this thread holds Yr and Yi of src for the 8
+  // src = SQ w + s.  After the two lane exchanges this thread holds Yr and Yi of src for the 8
   // columns coff .. coff+7 of each 32-column group (parts 0, 2, 1, 3 -> columns 0, 8, 16, 24).
   const int wq = warp & 3, we = warp >> 2;
-  const int part = lane >> 3, sl = lane & 7, src = 8 * wq + sl;
+  const int part = (lane / SQ) & 3, sl = lane % SQ, src = SQ * wq + sl;
   const int coff = 16 * (part & 1) + 8 * (part >> 1);
   const bool odd = (part & 1) != 0, up = part >= 2;
-  const bool live = r0 + src < nrhs;
+  const bool act = lane < 4 * SQ;   // (SQ = 4: the upper lanes of a quarter hold no rows)
+  const bool live = act && r0 + src < nrhs;
   const double2 *rgs = rg + (int64_t)(live ? r0 + src : 0) * vec_stride + s.ex0;
   float2 *stg = staging + (int64_t)(live ? r0 + src : 0) * stg_stride + s.soff;
   const bool pairs = ((s.soff | stg_stride | m) & 1) == 0;   // rows of the staging buffer start on 16 bytes
@@ -327,10 +339,10 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
   // V_0 = rho_0 (zero in the K padding columns m <= a < mp8)
   for (int g = we; g < ngrp; g += X3_E) {
     const int k0 = 32 * g + coff;
-    if (k0 < mp8) {
+    if (act && k0 < mp8) {
       float2 v[8];
       load_rho(s.ey0, k0, v);
-      put_v8(A1, A2, asbo, wq, sl, k0, v);
+      put_v8<SQ>(A1, A2, asbo, wq, sl, k0, v);
     }
     tc::fence_async_smem();
     tc::fence_before();
@@ -393,23 +405,23 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
       const int g = we + o * X3_E;
       if (g >= ngrp) break;
       const int k0 = 32 * g + coff;
-      const bool colok = k0 < mp8;
+      const bool colok = act && k0 < mp8;
       float v[32];
       tmem_ld32(dcol + (uint32_t)(32 * g), v);   // warp-collective
-      // hi + lo parts (lanes l, l ^ 8): keep 16 of the 32 columns
+      // hi + lo parts (lanes l, l ^ SQ): keep 16 of the 32 columns
       float h[16];
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
         const float x = odd ? v[c] : v[16 + c];
-        const float y = __shfl_xor_sync(0xffffffffu, x, 8);
+        const float y = __shfl_xor_sync(0xffffffffu, x, SQ);
         h[c] = (odd ? v[16 + c] : v[c]) + y;
       }
-      // real and imaginary parts (lanes l, l ^ 16): keep 8 columns, both parts
+      // real and imaginary parts (lanes l, l ^ 2 SQ): keep 8 columns, both parts
       float2 y8[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const float x = up ? h[c] : h[8 + c];
-        const float y = __shfl_xor_sync(0xffffffffu, x, 16);
+        const float y = __shfl_xor_sync(0xffffffffu, x, 2 * SQ);
         const float own = up ? h[8 + c] : h[c];
         y8[c] = up ? make_float2(y, own) : make_float2(own, y);
       }
@@ -423,7 +435,7 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
           nv[i] = nfwd ? cfms(lc, out[i], pre[o][i]) : cmul(lc, out[i]);
           if (a >= m) nv[i] = make_float2(0.f, 0.f);
         }
-        if (has_next) put_v8(A1, A2, asbo, wq, sl, k0, nv);
+        if (has_next) put_v8<SQ>(A1, A2, asbo, wq, sl, k0, nv);
         if (has_next) {
           tc::fence_async_smem();
           tc::fence_before();
@@ -456,25 +468,38 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
 
 // One CTA per SM (the two accumulators take all 512 tensor-memory columns); ring stages
 // as many as fit beside the A operands, at least two.
-cudaError_t launch_subst_x3(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
-                            int64_t stg_stride, cudaStream_t st) {
+template <int SQ>
+static cudaError_t launch_x3(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
+                             int64_t stg_stride, cudaStream_t st) {
   const int mp8max = (ctx->max_m + 7) & ~7;
-  if (mp8max > kMaxBoxWidthX3) return cudaErrorInvalidValue;
-  const int groups = (nrhs + X3_NR - 1) / X3_NR;
+  const int groups = (nrhs + 4 * SQ - 1) / (4 * SQ);
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   int ns = 2;
-  while (ns < 8 && subst_x3_smem(ns + 1, mp8max) <= (size_t)optin) ++ns;
-  size_t smem = subst_x3_smem(ns, mp8max);
+  while (ns < 8 && subst_x3_smem(SQ, ns + 1, mp8max) <= (size_t)optin) ++ns;
+  size_t smem = subst_x3_smem(SQ, ns, mp8max);
   if (smem > (size_t)optin) return cudaErrorInvalidValue;
   smem = std::max(smem, (size_t)optin / 2 + 1024);   // keeps a second CTA off the SM
-  cudaError_t e = allow_smem(k_subst_x3, smem);
+  cudaError_t e = allow_smem(k_subst_x3<SQ>, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(groups, ctx->nsub);
-  k_subst_x3<<<grid, X3_THREADS, smem, st>>>(ctx->d_subs, ctx->d_lpool, reinterpret_cast<const float *>(ctx->factor),
-                                             r, ctx->NX, vec_stride, reinterpret_cast<float2 *>(staging), stg_stride,
-                                             nrhs, ns, mp8max, ctx->d_status);
+  k_subst_x3<SQ><<<grid, X3_THREADS, smem, st>>>(ctx->d_subs, ctx->d_lpool, reinterpret_cast<const float *>(ctx->factor),
+                                                 r, ctx->NX, vec_stride, reinterpret_cast<float2 *>(staging), stg_stride,
+                                                 nrhs, ns, mp8max, ctx->d_status);
   return cudaGetLastError();
+}
+
+cudaError_t launch_subst_x3(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
+                            int64_t stg_stride, cudaStream_t st) {
+  if (((ctx->max_m + 7) & ~7) > kMaxBoxWidthX3) return cudaErrorInvalidValue;
+  // 16 or 32 right-hand sides per CTA: the shorter of the two launches, in waves of CTAs times the
+  // cycles of a step (17.6K and 22.5K at m = 176).  Measured (ms, 16 / 32 per CTA): 16 sources in 64
+  // boxes 3.27 / 4.00, 32 in 64 3.41 / 4.40, 40 in 196 10.9 / 10.3, 64 in 256 23.1 / 17.5.
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  auto waves = [&](int nr) { return ((int64_t)ctx->nsub * ((nrhs + nr - 1) / nr) + sms - 1) / sms; };
+  return 176 * waves(16) <= 225 * waves(32) ? launch_x3<4>(ctx, r, nrhs, vec_stride, staging, stg_stride, st)
+              : launch_x3<8>(ctx, r, nrhs, vec_stride, staging, stg_stride, st);
 }
 
 }  // namespace hd

@@ -17,7 +17,7 @@
 //
 // Kernels: k_dots (block partial sums of V^H w, w held in registers), k_reduce
 // (fixed-order sum of the partials: deterministic), k_update (w = base + sgn V c,
-// optionally with block partials of ||w||^2), and one-thread-per-right-hand-side
+// optionally with block partials of ||w||^2), and one-warp-per-right-hand-side
 // kernels for the O(restart) Hessenberg/Givens/triangular work.  The host reads
 // 32 bytes per right-hand side and Arnoldi step to decide whether to stop.
 #include <algorithm>

@@ -92,19 +92,25 @@ struct OpArgs {
 //
 // Outside the PML every alpha is 1 and a row is x_W + x_E + x_S + x_N + cc x_C with the stored
 // centre cc = h^2 k^2 - 4: few bytes per cell, and FP64 runs at 1/64 of FP32, so the FP64 pipe
-// bounds it (a third above the time of its bytes).  The sum is taken as
-// (x_W + x_N) + (x_S + x_E): x_S + x_E of cell (i, j) is x_W + x_N of cell (i + 1, j - 1), so a
-// warp that walks down the grid forms each pair once and passes it to the lane on its left, and
-// a cell costs two additions and one FMA per component instead of three and one.  A warp takes
-// ST_COLS columns (its last lane only forms pairs) and `R` rows; every entry of x is loaded once
-// per tile.  The tiles fill the part outside the PML from its lower corner; the frame around
-// them (the PML and what is left of a tile) takes the general form, a thread per cell.
-// 4096^2: 300 -> 224 us (FP64 pipe at 1.7 of its 2 lanes a cycle and SM); 1024^2: 36 -> 25 us.
+// bounds it (two thirds above the time of its bytes).  The sum is taken as
+// (x_S + x_E + cc x_C) + (x_W + x_N): x_S + x_E of cell (i, j) is x_W + x_N of cell (i + 1, j - 1),
+// so a warp that walks down the grid forms each pair once and passes it to the lane on its left,
+// and a cell costs two additions and one FMA per component instead of three and one.  The centre
+// joins one pair before the pairs meet: for a wave the two halves nearly cancel, and their sum
+// is exact or close to it, where x_W + x_N + x_S + x_E would be rounded at four times the wave's size
+// first.  (Error against extended precision on waves of 10 to 20 cells, relative to the four
+// neighbours added one by one to cc x_C: 1.01 to 1.07, with the four summed first 1.35 to 1.49;
+// on white noise 0.76.)
+// A warp takes ST_COLS columns (its last lane only forms pairs) and `R` rows; every entry of x is
+// loaded once per tile.  The tiles fill the part outside the PML from its lower corner; the frame
+// around them (the PML and what is left of a tile) takes the general form, a thread per cell.
+// 4096^2: 300 -> 225 us (FP64 pipe 78 % busy); 1024^2: 36 -> 25 us.
 constexpr int ST_COLS = 31, ST_WARPS = 8;
 
-template <int MODE> __device__ __forceinline__ double2 stencil_end(double cc, double2 xc, double2 s, double2 b) {
-  if (MODE == 1) return make_double2(__fma_rn(-cc, xc.x, add_rn(b.x, -s.x)), __fma_rn(-cc, xc.y, add_rn(b.y, -s.y)));
-  return make_double2(__fma_rn(cc, xc.x, s.x), __fma_rn(cc, xc.y, s.y));
+// p = x_S + x_E, q = x_W + x_N (in a tile p is there a row before q)
+template <int MODE> __device__ __forceinline__ double2 stencil_end(double cc, double2 xc, double2 p, double2 q, double2 b) {
+  const double2 y = cadd(make_double2(__fma_rn(cc, xc.x, p.x), __fma_rn(cc, xc.y, p.y)), q);
+  return MODE == 1 ? csub(b, y) : y;
 }
 
 // One cell anywhere in the grid.
@@ -117,7 +123,7 @@ __device__ __forceinline__ void stencil_cell(const OpArgs &a, const double2 *__r
   const double2 xw = i > 0 ? x[idx - 1] : zero, xe = i + 1 < a.NX ? x[idx + 1] : zero;
   const double2 xs = j > 0 ? x[idx - a.NX] : zero, xn = j + 1 < a.NY ? x[idx + a.NX] : zero;
   if (i >= a.npml && i < a.NX - a.npml && j >= a.npml && j < a.NY - a.npml) {
-    y[idx] = stencil_end<MODE>(a.cc[idx], xc, cadd(cadd(xw, xn), cadd(xs, xe)), MODE == 1 ? b[idx] : zero);
+    y[idx] = stencil_end<MODE>(a.cc[idx], xc, cadd(xs, xe), cadd(xw, xn), MODE == 1 ? b[idx] : zero);
     return;
   }
   const double2 a1 = a.ax_c[i], a2 = a.ay_c[j];
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS) k_stencil(OpArgs a, StencilTile
     const double2 bv = MODE == 1 ? pb[0] : make_double2(0.0, 0.0);
     const double2 e = shfl_down1(d);   // x_S + x_E of this cell
     d = cadd(west(p, xc), xn);
-    if (lane < ST_COLS) py[0] = stencil_end<MODE>(cc, xc, cadd(d, e), bv);
+    if (lane < ST_COLS) py[0] = stencil_end<MODE>(cc, xc, e, d, bv);
     xc = xn;
     p += a.NX;
     pc += a.NX;

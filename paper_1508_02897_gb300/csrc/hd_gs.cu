@@ -111,8 +111,7 @@ __device__ __forceinline__ void gs_produce(const GsRing &g, int64_t n, int S, in
     atomicOr(status, ST_TIMEOUT);
   }
   // no copy may still be landing in shared memory when the CTA exits
-  for (uint32_t k = issued > (uint32_t)GS_NS ? issued - GS_NS : 0u; k < issued; ++k)
-    tc::bar_wait(&g.full[k % GS_NS], (k / GS_NS) & 1u, g.abort_flag);
+  tc::ring_drain(g.full, issued, GS_NS);
 }
 
 // Consumer side of one tile: wait for it (once per thread; a failed wait flags the abort).

@@ -24,6 +24,7 @@
 // 3 x 3, in practice 2 x 2) boxes whose extent covers the cell: deterministic,
 // no atomics.
 #include "hd_internal.cuh"
+#include "hd_tc.cuh"
 
 namespace hd {
 
@@ -177,8 +178,7 @@ k_subst(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, const
         atomicOr(status, ST_TIMEOUT);
       }
       // no copy may still be landing in shared memory when the CTA exits
-      for (int64_t it = max((int64_t)0, issued - NS); it < issued; ++it)
-        mbar_wait(&full[it % NS], (uint32_t)((it / NS) & 1), abort_flag);
+      tc::ring_drain(full, issued, NS);
     }
     return;
   }

@@ -410,8 +410,7 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
         atomicOr(status, ST_TIMEOUT);
       }
       // no copy may still be landing in shared memory when the CTA exits
-      for (int it = max(0, issued - NS); it < issued; ++it)
-        tc::bar_wait(&pf[it % NS], (uint32_t)((it / NS) & 1), abort_flag);
+      tc::ring_drain(pf, issued, NS);
     }
   } else {
     // ---------------- consumer warps; thread a < m of vector group vg owns output a of the

@@ -29,6 +29,7 @@
 // Every wait is bounded (flag ST_TIMEOUT and unwind); tensor memory is released
 // only after a final commit confirms that no MMA is in flight.
 #include "hd_internal.cuh"
+#include "hd_tc.cuh"
 
 namespace hd {
 
@@ -117,11 +118,11 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
 }  // namespace
 
 // Shared memory: A1, A2 [144 * mp8max bytes each] | ring [NS][64 * mp8max] | Ys [mp8max][33] floats |
-// full[NS] | empty[NS] | dfull | bready | fin | tmem address | abort flag.  The M = 64 reads
+// full[NS] | empty[NS] | dfull | bready | fin | edone | tmem address | abort flag.  The M = 64 reads
 // of A2 run 144 * mp8max bytes past its end (rows 32..63, never used), into the ring and Ys.
 size_t subst_tc_smem(int ns, int mp8max) {
   return 2 * (size_t)kBLbo * mp8max + (size_t)ns * 64 * mp8max + (size_t)kYsLd * 4 * mp8max +
-         (2 * (size_t)ns + 3) * 8 + 16;
+         (2 * (size_t)ns + 4) * 8 + 16;
 }
 
 __global__ void __launch_bounds__(TC_THREADS, 2)
@@ -142,7 +143,8 @@ k_subst_tc(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
   uint64_t *dfull = empty + NS;
   uint64_t *bready = dfull + 1;
   uint64_t *fin = bready + 1;
-  uint32_t *tholder = reinterpret_cast<uint32_t *>(fin + 1);
+  uint64_t *edone = fin + 1;
+  uint32_t *tholder = reinterpret_cast<uint32_t *>(edone + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tholder + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t bsbo = kBLbo * (uint32_t)(mp8max / 4);   // A1/A2: bytes between 8-row groups
@@ -155,6 +157,7 @@ k_subst_tc(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
     tbar_init(dfull, 1);
     tbar_init(bready, TC_EPI);
     tbar_init(fin, 1);
+    tbar_init(edone, TC_EPI);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -199,8 +202,8 @@ k_subst_tc(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
         *abort_flag = 1;
         atomicOr(status, ST_TIMEOUT);
       }
-      for (int64_t it = max((int64_t)0, issued - NS); it < issued; ++it)
-        tbar_wait(&full[it % NS], (uint32_t)((it / NS) & 1), abort_flag);
+      // no copy may still be landing in shared memory when the CTA exits
+      tc::ring_drain(full, issued, NS);
     }
     return;
   }
@@ -234,8 +237,8 @@ k_subst_tc(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
         atomicOr(status, ST_TIMEOUT);
       }
       mma_commit(fin);                          // arrives once every MMA issued above is done
-      tbar_wait(fin, 0, abort_flag);
-      tbar_wait(bready, (uint32_t)(nsteps & 1), abort_flag);   // epilogue done reading TMEM
+      tc::bar_drain(fin, 0);
+      tc::bar_drain(edone, 0);                  // the epilogue has finished reading tensor memory
     }
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -375,6 +378,8 @@ k_subst_tc(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     tbar_arrive(bready);
   }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tbar_arrive(edone);   // (on a timeout too)
 }
 
 // Stages of the ring: as many as fit beside the B operands for the CTAs that

@@ -260,8 +260,7 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
         atomicOr(status, ST_TIMEOUT);
       }
       // no copy may still be landing when the CTA exits
-      for (int it = max(0, issued - NS); it < issued; ++it)
-        tc::bar_wait(&full[it % NS], (uint32_t)((it / NS) & 1), abort_flag);
+      tc::ring_drain(full, issued, NS);
     }
     return;
   }
@@ -303,8 +302,8 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
         atomicOr(status, ST_TIMEOUT);
       }
       tc::mma_commit(fin);                          // arrives once every MMA issued above is done
-      tc::bar_wait(fin, 0, abort_flag);
-      tc::bar_wait(edone, 0, abort_flag);           // the epilogue has finished reading tensor memory
+      tc::bar_drain(fin, 0);
+      tc::bar_drain(edone, 0);                      // the epilogue has finished reading tensor memory
     }
     __syncwarp();
     tc::fence_after();

@@ -53,6 +53,27 @@ __device__ __forceinline__ bool bar_spin(uint64_t *bar, uint32_t parity, volatil
   return false;
 }
 
+// Before a CTA gives up its shared or tensor memory, what it has in flight (bulk copies, MMAs,
+// another warp's tensor-memory reads) has to land.  These waits come after a timeout too, when
+// the abort flag is already set, so they do not look at it: kWaitLimit polls bound them.
+template <typename Poll> __host__ __device__ __forceinline__ bool drain(Poll landed) {
+  for (uint32_t it = 0; it < kWaitLimit; ++it)
+    if (landed()) return true;
+  return false;
+}
+// The copies still in flight in a ring of ns stages after `issued` copies: at most one per stage,
+// copy k on stage k % ns in its lap k / ns.  landed(stage, parity): that lap's copy is in.
+template <typename Poll> __host__ __device__ __forceinline__ void drain_ring(int64_t issued, int ns, Poll landed) {
+  for (int64_t k = issued > ns ? issued - ns : 0; k < issued; ++k)
+    drain([&]() { return landed((int)(k % ns), (uint32_t)((k / ns) & 1)); });
+}
+__device__ __forceinline__ void bar_drain(uint64_t *bar, uint32_t parity) {
+  drain([&]() { return bar_try(bar, parity); });
+}
+__device__ __forceinline__ void ring_drain(uint64_t *full, int64_t issued, int ns) {
+  drain_ring(issued, ns, [&](int stage, uint32_t parity) { return bar_try(&full[stage], parity); });
+}
+
 // Shared-memory matrix descriptor of the no-swizzle K-major layout: start address,
 // leading byte offset (between core matrices adjacent along K), stride byte offset
 // (between 8-row groups along M or N), descriptor version 1.

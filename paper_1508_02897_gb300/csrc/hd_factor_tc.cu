@@ -86,7 +86,7 @@ constexpr size_t kOffG = kOffY + sizeof(float2) * FX_ROWS * CLD;
 constexpr size_t kOffL = kOffG + sizeof(float2) * 2 * FX_KP * FX_KP;
 constexpr size_t kOffD = kOffL + sizeof(float2) * FX_ROWS;
 constexpr size_t kOffM = kOffD + sizeof(float2) * 3 * FX_ROWS;
-constexpr size_t kSmem = kOffM + 32;
+constexpr size_t kSmem = kOffM + 48;
 
 // (x0, x1) = h + m + l piecewise, BF16 pieces rounded to nearest (each remainder is
 // exact in FP32), two values per conversion instruction; the pieces come packed as
@@ -184,7 +184,8 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   float2 *dS = reinterpret_cast<float2 *>(smem_raw + kOffD);   // [3][FX_ROWS] band entries of the next row's D
   float2 *lS = reinterpret_cast<float2 *>(smem_raw + kOffL);   // [FX_ROWS] coupling of the next row
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem_raw + kOffM);
-  uint32_t *tholder = reinterpret_cast<uint32_t *>(mbar + 2);
+  uint64_t *fin = mbar + 2;   // the release of tensor memory after a timeout
+  uint32_t *tholder = reinterpret_cast<uint32_t *>(fin + 1);
   volatile int *sflag = reinterpret_cast<volatile int *>(tholder + 1);
   volatile int *abort_flag = sflag + 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -192,6 +193,7 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   if (tid == 0) {
     tc::bar_init(mbar, 1);
     tc::bar_init(mbar + 1, 1);
+    tc::bar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -672,9 +674,10 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   tc::fence_before();
   __syncthreads();
   if (!alive && issuer) {
-    tc::mma_commit(mbar);   // arrives when every MMA issued so far has completed
-    volatile int never = 0;
-    tc::bar_wait(mbar, nphase & 1u, &never);
+    // (on a barrier of its own: a panel's barrier that timed out is still in the phase the count has
+    // left behind, and the parity of the next one would pass at once)
+    tc::mma_commit(fin);   // arrives when every MMA issued so far has completed
+    tc::bar_drain(fin, 0);
   }
   __syncthreads();
   tc::fence_after();

@@ -84,3 +84,14 @@ def test_tensor_memory_is_released_after_its_last_use(name):
     tail = s[s.index("mma_commit(fin)"):s.index("tcgen05.dealloc")]
     assert "tc::bar_drain(fin, 0);" in tail and "tc::bar_drain(edone, 0);" in tail and "abort_flag" not in tail
     assert len(re.findall(r"arrive\(edone\)", s)) == 1
+
+
+def test_factorisation_releases_tensor_memory_after_its_last_mma():
+    """After a timeout the last commit goes to a barrier that no other wait uses: the parity of a
+    panel's barrier that never completed would pass at once."""
+    s = _source("hd_factor_tc.cu")
+    tail = s[s.index("release tensor memory"):s.index("tcgen05.dealloc")]
+    bar = re.search(r"tc::mma_commit\((\w+)\)", tail).group(1)
+    assert f"tc::bar_drain({bar}, 0)" in tail
+    assert len(re.findall(rf"tc::mma_commit\({bar}\)", s)) == 1 and len(re.findall(rf"bar_init\({bar}, 1\)", s)) == 1
+    assert not re.search(rf"(wait|spin)\({bar}\b", s)

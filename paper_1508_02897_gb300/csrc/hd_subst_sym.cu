@@ -35,7 +35,9 @@
 //
 // Hazards of the cluster form.  Received group sums sit in two buffers (even and odd
 // steps): a CTA sends step t + 2 only after it has every sum of step t + 1, which the
-// receiver sent after it was done with step t.  Row j of the staging buffer is written by
+// receiver sent after it was done with step t.  A thread that gave up a wait sends no more (it
+// would run ahead of that bound, and of what an mbarrier can count), so the other CTAs give up
+// too.  Row j of the staging buffer is written by
 // one CTA and read by all in the back substitution: a release / acquire pair at cluster
 // scope (barrier `turn`) separates the two sweeps, and x_j replaces w_j one step late, when
 // the other CTAs' sums of the step after prove that they have used w_j.
@@ -85,6 +87,10 @@ __device__ __forceinline__ void cluster_send(uint32_t dst, double2 v, uint32_t b
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
                "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar)
                : "memory");
+}
+// About a millisecond: a thousand times what a store into another CTA's shared memory takes.
+__device__ __forceinline__ void settle() {
+  for (const long long t0 = clock64(); clock64() - t0 < 2000000;) {}
 }
 // Bounded wait with acquire semantics at cluster scope (the phase is completed by other CTAs).
 __device__ __forceinline__ bool wait_cluster(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {
@@ -604,10 +610,10 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
           for (int q = 0; q < NV; ++q)
 #pragma unroll
             for (int d = 1; d < K; ++d)
-              cluster_send(peer_pb[d] + (uint32_t)(((par * SYM_GROUPS + gi) * NR + q) * mpmax * (int)sizeof(T)),
-                           p[gi][q], peer_bar[d] + (uint32_t)par * 8u);
+              if (ok) cluster_send(peer_pb[d] + (uint32_t)(((par * SYM_GROUPS + gi) * NR + q) * mpmax * (int)sizeof(T)),
+                                   p[gi][q], peer_bar[d] + (uint32_t)par * 8u);
         }
-        if (K > 1 && tid == 0)
+        if (K > 1 && tid == 0 && ok)
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::su32(&xbar[par])),
                        "r"((uint32_t)((SYM_GROUPS - GPC) * NR * m * (int)sizeof(T)))
                        : "memory");
@@ -656,7 +662,12 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
       for (int q = 0; q < NV; ++q)
         if (q < nlive) stga[q * stg_stride] = x[q];   // x_0
   }
-  if (K > 1) cluster_sync_all();   // no CTA leaves while another may still write into its shared memory
+  if (K > 1) {
+    cluster_sync_all();   // no CTA leaves while another may still write into its shared memory
+    // st.async is not ordered by the barrier.  Where no wait failed, every sum sent here has been
+    // waited for; else some may still be on their way, and the CTA stays until they have landed
+    if (*abort_flag) settle();
+  }
 }
 
 // ---------------------------------------------------------------- launch

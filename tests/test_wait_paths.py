@@ -95,3 +95,16 @@ def test_factorisation_releases_tensor_memory_after_its_last_mma():
     assert f"tc::bar_drain({bar}, 0)" in tail
     assert len(re.findall(rf"tc::mma_commit\({bar}\)", s)) == 1 and len(re.findall(rf"bar_init\({bar}, 1\)", s)) == 1
     assert not re.search(rf"(wait|spin)\({bar}\b", s)
+
+
+def test_cluster_exchange_stops_after_a_timeout():
+    """The CTAs of a cluster stay within two steps of each other only while every wait succeeds: a
+    thread that gave up neither sends sums nor arms the barrier for more, and its CTA outlasts the
+    sums that are still on their way to it."""
+    s = _source("hd_subst_sym.cu")
+    body = s[s.index("k_subst_sym("):s.index("static int sm_count()")]
+    sends = re.findall(r"(.*)\bcluster_send\(", body)
+    assert sends and all("if (ok)" in line for line in sends)
+    arms = re.findall(r"if \((K > 1 && tid == 0[^)]*)\)\s*asm volatile\(\"mbarrier\.arrive\.expect_tx", body)
+    assert arms == ["K > 1 && tid == 0 && ok"]
+    assert "if (*abort_flag) settle();" in body[body.rindex("cluster_sync_all();"):]

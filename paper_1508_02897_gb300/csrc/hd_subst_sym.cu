@@ -35,9 +35,9 @@
 //
 // Hazards of the cluster form.  Received group sums sit in two buffers (even and odd
 // steps): a CTA sends step t + 2 only after it has every sum of step t + 1, which the
-// receiver sent after it was done with step t.  A thread that gave up a wait sends no more (it
-// would run ahead of that bound, and of what an mbarrier can count), so the other CTAs give up
-// too.  Row j of the staging buffer is written by
+// receiver sent after it was done with step t.  A thread that gave up a wait leaves its vector
+// work, and with it the exchange (it would run ahead of that bound, and of what an mbarrier can
+// count), so the other CTAs give up too.  Row j of the staging buffer is written by
 // one CTA and read by all in the back substitution: a release / acquire pair at cluster
 // scope (barrier `turn`) separates the two sweeps, and x_j replaces w_j one step late, when
 // the other CTAs' sums of the step after prove that they have used w_j.
@@ -425,7 +425,7 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
     const int vg = VG > 1 && tid >= vspan ? 1 : 0;
     const int a = tid - vg * vspan, A = a >> 4, q0 = vg * NV;
     const int gx = s.ex0 + a;
-    const bool vec = a < m;
+    bool vec = a < m;   // has vector work (until a wait fails)
     const bool ownx = vec && gx >= s.ox0 && gx < s.ox1;
     const bool writer = vec && (K == 1 || (uint32_t)((a >> 5) % K) == rank);
     const int nlive = nrhs - r0 - q0;   // right-hand sides q < nlive exist
@@ -441,7 +441,7 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
     }
     bool ok = true;
     auto fail = [&]() {
-      ok = false;
+      ok = vec = false;
       *abort_flag = 1;
       atomicOr(status, ST_TIMEOUT);
     };
@@ -610,10 +610,10 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
           for (int q = 0; q < NV; ++q)
 #pragma unroll
             for (int d = 1; d < K; ++d)
-              if (ok) cluster_send(peer_pb[d] + (uint32_t)(((par * SYM_GROUPS + gi) * NR + q) * mpmax * (int)sizeof(T)),
-                                   p[gi][q], peer_bar[d] + (uint32_t)par * 8u);
+              cluster_send(peer_pb[d] + (uint32_t)(((par * SYM_GROUPS + gi) * NR + q) * mpmax * (int)sizeof(T)),
+                           p[gi][q], peer_bar[d] + (uint32_t)par * 8u);
         }
-        if (K > 1 && tid == 0 && ok)
+        if (K > 1 && tid == 0)
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::su32(&xbar[par])),
                        "r"((uint32_t)((SYM_GROUPS - GPC) * NR * m * (int)sizeof(T)))
                        : "memory");

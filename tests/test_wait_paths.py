@@ -103,8 +103,8 @@ def test_cluster_exchange_stops_after_a_timeout():
     sums that are still on their way to it."""
     s = _source("hd_subst_sym.cu")
     body = s[s.index("k_subst_sym("):s.index("static int sm_count()")]
-    sends = re.findall(r"(.*)\bcluster_send\(", body)
-    assert sends and all("if (ok)" in line for line in sends)
-    arms = re.findall(r"if \((K > 1 && tid == 0[^)]*)\)\s*asm volatile\(\"mbarrier\.arrive\.expect_tx", body)
-    assert arms == ["K > 1 && tid == 0 && ok"]
+    assert "ok = vec = false;" in body[body.index("auto fail"):]
+    work = body[body.rindex("if (vec) {"):]   # the vector work of a step, which ends with the thread's first failed wait
+    for op in ("cluster_send(", "mbarrier.arrive.expect_tx"):
+        assert body.count(op) == work.count(op) > 0
     assert "if (*abort_flag) settle();" in body[body.rindex("cluster_sync_all();"):]

@@ -441,7 +441,8 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
     }
     bool ok = true;
     auto fail = [&]() {
-      ok = vec = false;
+      ok = false;
+      if (K > 1) vec = false;
       *abort_flag = 1;
       atomicOr(status, ST_TIMEOUT);
     };

@@ -204,13 +204,13 @@ enum { LAY_FULL = 0, LAY_SYM = 1, LAY_TC = 2, LAY_TC3 = 3 };
 
 // Symmetric tile storage: the upper 16 x 16 tiles of an m x m block, column by column
 // (tile (I, J) at J(J+1)/2 + I, I <= J < mt = ceil(m / 16)).  The substitution takes them in
-// segments: up to SYM_SEG tiles one above the other, (3k .. 3k + 2, J); segments are numbered
+// segments: up to `seg` (1 or 3) tiles one above the other, (3k .. 3k + 2, J); segments are numbered
 // column by column and cut into SYM_GROUPS groups of consecutive ones, whose sums are formed
 // apart (SymMap: the numbering, shared by the kernel and its tables).
-constexpr int SYM_SEG = 3, SYM_GROUPS = 4;
+constexpr int SYM_GROUPS = 4;
 struct SymMap {
-  int mt, nt, nseg, base, rem;
-  __host__ __device__ explicit SymMap(int m) {
+  int seg, mt, nt, nseg, base, rem;
+  __host__ __device__ SymMap(int m, int seg_) : seg(seg_) {
     mt = (m + 15) / 16;
     nt = mt * (mt + 1) / 2;
     nseg = col_seg(mt);
@@ -218,9 +218,10 @@ struct SymMap {
     rem = nseg - base * SYM_GROUPS;
   }
   // first segment of column J: the columns before it have 1, 1, 1, 2, 2, 2, 3, ... segments
-  static __host__ __device__ int col_seg(int J) {
-    const int q = J / SYM_SEG, r = J - q * SYM_SEG;
-    return SYM_SEG * q * (q + 1) / 2 + r * (q + 1);
+  __host__ __device__ int col_seg(int J) const {
+    if (seg == 1) return J * (J + 1) / 2;
+    const int q = J / 3, r = J - q * 3;
+    return 3 * q * (q + 1) / 2 + r * (q + 1);
   }
   __host__ __device__ int group_start(int g) const { return g * base + (g < rem ? g : rem); }   // in segments
   __host__ __device__ int group_of(int s) const {
@@ -231,7 +232,7 @@ struct SymMap {
   __host__ __device__ void segment(int s, int &I, int &J) const {
     J = 0;
     while (J < mt && col_seg(J + 1) <= s) ++J;
-    I = SYM_SEG * (s - col_seg(J));
+    I = seg * (s - col_seg(J));
   }
   __host__ __device__ int first_tile(int s) const {
     int I, J;

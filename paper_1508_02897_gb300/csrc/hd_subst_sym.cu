@@ -4,13 +4,13 @@
 // y_J += T^T v_I.
 //
 // Order of the sum.  The tiles lie column by column and are taken in segments of up to
-// three tiles of one column J (SymMap in hd_internal.cuh), the segments in SYM_GROUPS
-// groups.  One warp takes a segment: each lane holds 2 x 4 entries of every tile in
+// three tiles of one column J (one tile in complex FP64 where no box is wider than 64; SymMap in
+// hd_internal.cuh), the segments in SYM_GROUPS groups.  One warp takes a segment: each lane holds 2 x 4 entries of every tile in
 // registers and forms both products from that one read; the column products T^T v_I add up
 // over the segment, the row products T v_J are summed tile by tile, and the 16 sums of each
 // go to a slot of their own in shared memory.  One thread per output then adds, group by
 // group, the row slots (J ascending) and the column slots (segments ascending), and the
-// group sums in order.  That order depends on the block's width alone: a launch may spread
+// group sums in order.  That order depends on the widths of the boxes alone: a launch may spread
 // the groups over K CTAs of a cluster, over P sets of warps, and may run one or several
 // right-hand sides per CTA, with bitwise the same result.
 //
@@ -45,6 +45,7 @@
 #include <type_traits>
 
 #include "hd_internal.cuh"
+#include "hd_sym_shape.cuh"
 #include "hd_tc.cuh"
 
 namespace hd {
@@ -210,10 +211,9 @@ template <typename T> __device__ __forceinline__ decltype(T::x) reduce_cols(cons
 }
 
 // ---------------------------------------------------------------- launch shape
-// Warps of a set, a segment each per round: 7 in complex FP32 (two sets and a producer make 15
-// warps, which leaves 128 registers a thread), 8 in complex FP64, whose products keep the four
-// FP64 pipes of the SM equally busy only if the warps divide by four.
-template <typename R> constexpr int set_warps() { return sizeof(R) == 4 ? 7 : 8; }
+// Warps of a set, a segment each per round (SW): 7 in complex FP32 (two sets and a producer make
+// 15 warps, which leaves 128 registers a thread), 8 in complex FP64, whose products keep the four
+// FP64 pipes of the SM equally busy only if the warps divide by four, 3 in the small form.
 constexpr int MAXTERM = 8;               // sums of one output in one group (boxes up to 256 wide)
 
 // Rounds of a group of n segments, at most `spr` (<= the set's warps) a round; round c takes the segments
@@ -222,10 +222,10 @@ __host__ __device__ __forceinline__ int sym_rounds(int n, int spr) { return (n +
 
 // Tiles of the largest round (one ring stage) of any box up to mt tiles wide: a narrower box
 // may have fewer rounds, and so larger ones.
-static int sym_stage_tiles(int mt, int spr) {
+static int sym_stage_tiles(int mt, int spr, int seg) {
   int most = 1;
   for (int t = 1; t <= mt; ++t) {
-    const SymMap map(16 * t);
+    const SymMap map(16 * t, seg);
     for (int g = 0; g < SYM_GROUPS; ++g) {
       const int b = map.group_start(g), n = map.group_start(g + 1) - b, nr = sym_rounds(n, spr);
       for (int c = 0; c < nr; ++c)
@@ -243,8 +243,8 @@ struct SymSmem {
   int nslot, maxround;
 };
 template <typename R, typename S>
-__host__ __device__ inline SymSmem sym_smem(int ns, int stage_tiles, int spr, int mp, int K, int P, int nr) {
-  const SymMap map(mp);
+__host__ __device__ inline SymSmem sym_smem(int ns, int stage_tiles, int spr, int mp, int K, int P, int nr, int sw, int seg) {
+  const SymMap map(mp, seg);
   SymSmem L;
   L.nslot = map.nt + map.nseg + 1;
   L.maxround = sym_rounds(map.base + (map.rem > 0), spr) * (SYM_GROUPS / (K * P));   // rounds of a set per step
@@ -254,7 +254,7 @@ __host__ __device__ inline SymSmem sym_smem(int ns, int stage_tiles, int spr, in
   L.terms = L.pb + (K > 1 ? 2 * (size_t)SYM_GROUPS * nr * mp * 2 * sizeof(R) : 0);
   L.rounds = L.terms + (size_t)SYM_GROUPS * map.mt * MAXTERM * sizeof(uint16_t);
   L.items = L.rounds + (size_t)P * (L.maxround + 1) * sizeof(uint32_t);
-  L.bars = (L.items + (size_t)P * L.maxround * set_warps<R>() * sizeof(uint32_t) + 15) & ~(size_t)15;
+  L.bars = (L.items + (size_t)P * L.maxround * sw * sizeof(uint32_t) + 15) & ~(size_t)15;
   L.total = L.bars + (2 * (size_t)P * ns + 3) * sizeof(uint64_t) + 16;
   return L;
 }
@@ -264,26 +264,29 @@ __host__ __device__ inline SymSmem sym_smem(int ns, int stage_tiles, int spr, in
 // One cluster of K CTAs per (box, NR right-hand sides); the P sets of a CTA walk
 // SYM_GROUPS / (K P) groups each, one after another.  The vector work of a step is spread
 // over VG groups of warps, NR / VG right-hand sides each.
-template <typename R, typename S, int K, int P, int NR, int VG>
-__global__ void __launch_bounds__((P * set_warps<R>() + 1) * 32, sizeof(R) == 8 && K == 1 && NR == 1 ? 2 : 1)
+template <typename R, typename S, int K, int P, int NR, int VG, int SW, int PER_SM>
+__global__ void __launch_bounds__((P * SW + 1) * 32, PER_SM)
 k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
             const S *__restrict__ factor, const double2 *__restrict__ rg, int NX, int64_t vec_stride,
-            C<R> *__restrict__ staging, int64_t stg_stride, int nrhs, int NS, int ST, int SPR, int mpmax, int32_t *status) {
+            C<R> *__restrict__ staging, int64_t stg_stride, int nrhs, int NS, int ST, int SPR, int seg_tiles, int mpmax, int32_t *status) {
   using T = C<R>;
   using O = Ops<R>;
   using Vec = typename O::Vec;
   using Acc = typename O::Acc;
-  constexpr int SW = set_warps<R>(), PW = P * SW, CT = PW * 32;
+  constexpr int PW = P * SW, CT = PW * 32;
+  constexpr bool SMALL = PER_SM > 2;
   constexpr int NV = NR / VG;                          // right-hand sides of a vector thread
   constexpr int GPC = SYM_GROUPS / K, GPS = GPC / P;   // groups per CTA and per set
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const SubDev s = subs[blockIdx.y];
   const int m = s.ex, rows = s.ey;
-  const SymMap map(m);
+  const int SEG = sizeof(R) == 4 ? 3 : seg_tiles;   // (a constant where it can be)
+  const SymMap map(m, SEG);
   const int mt = map.mt, nt = map.nt;
   const uint32_t rank = K > 1 ? cluster_rank() : 0u;
   const int r0 = (int)(blockIdx.x / K) * NR;
-  const SymSmem L = sym_smem<R, S>(NS, ST, SPR, mpmax, K, P, NR);
+  const int nq = SMALL ? min(NR, nrhs - r0) : NR;   // right-hand sides to form products for
+  const SymSmem L = sym_smem<R, S>(NS, ST, SPR, mpmax, K, P, NR, SW, SEG);
   S *ring = reinterpret_cast<S *>(smem_raw);
   T *vs = reinterpret_cast<T *>(smem_raw + L.vs);
   R *slots = reinterpret_cast<R *>(smem_raw + L.slots);
@@ -297,7 +300,19 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
   uint64_t *turn = xbar + 2;
   volatile int *abort_flag = reinterpret_cast<volatile int *>(turn + 1);
   const int qstride = L.nslot * 32;   // slots of one right-hand side
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int warp = threadIdx.x >> 5;
+  if constexpr (SMALL && sizeof(R) == 8) {
+    // (FP64 runs at the rate of each quarter of the SM: the roles turn with the CTA's place on the SM, or
+    // the producers and the longest segments of its CTAs would meet on one quarter)
+    if (threadIdx.x == 0) {
+      uint32_t w;
+      asm volatile("mov.u32 %0, %%warpid;" : "=r"(w));
+      abort_flag[1] = (int)(w >> 2);
+    }
+    __syncthreads();
+    warp = (warp + abort_flag[1]) % (PW + 1);
+  }
+  const int lane = threadIdx.x & 31, tid = warp * 32 + lane;
   if (tid == 0) {
     for (int q = 0; q < P * NS; ++q) {
       tc::bar_init(&full[q], 1);
@@ -328,7 +343,7 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
   auto make_item = [&](int seg, int t0) {
     int I, J;
     map.segment(seg, I, J);
-    return (uint32_t)I | (uint32_t)J << 5 | (uint32_t)min(SYM_SEG, J - I + 1) << 10 |
+    return (uint32_t)I | (uint32_t)J << 5 | (uint32_t)min(SEG, J - I + 1) << 10 |
            (uint32_t)(J * (J + 1) / 2 + I - t0) << 12 | (uint32_t)seg << 17;
   };
   for (int i = tid; i < P * (L.maxround + 1); i += CT + 32) {
@@ -341,7 +356,7 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
     }
     rounds[i] = v;
   }
-  if constexpr (K == 1 && (sizeof(R) == 8 || NR > 1)) {
+  if constexpr (K == 1 && (SMALL || sizeof(R) == 8 || NR > 1)) {
     // bound by arithmetic: a segment goes to the free warp of the round whose quarter of the SM
     // (warp % 4) has the fewest products so far (lane = warp; the busiest quarter then has 2 to
     // 10 % more than the mean, up to 55 % when they are dealt out in order: 14.7 -> 13.5 ms per
@@ -379,12 +394,14 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
     const int g = i / mt, A = i - g * mt;
     int n = 0;
     for (int J = A; J < mt; ++J)
-      if (map.group_of(SymMap::col_seg(J) + A / SYM_SEG) == g) terms[i * MAXTERM + n++] = (uint16_t)((J * (J + 1) / 2 + A) * 32);
-    for (int k = 0; SYM_SEG * k < A; ++k)
-      if (map.group_of(SymMap::col_seg(A) + k) == g) terms[i * MAXTERM + n++] = (uint16_t)((nt + SymMap::col_seg(A) + k) * 32);
+      if (map.group_of(map.col_seg(J) + (SEG == 1 ? A : A / 3)) == g) terms[i * MAXTERM + n++] = (uint16_t)((J * (J + 1) / 2 + A) * 32);
+    for (int k = 0; SEG * k < A; ++k)
+      if (map.group_of(map.col_seg(A) + k) == g) terms[i * MAXTERM + n++] = (uint16_t)((nt + map.col_seg(A) + k) * 32);
     for (; n < MAXTERM; ++n) terms[i * MAXTERM + n] = (uint16_t)((nt + map.nseg) * 32);
   }
   for (int i = tid; i < NR * 32; i += CT + 32) slots[(i >> 5) * qstride + (nt + map.nseg) * 32 + (i & 31)] = (R)0;
+  if (SMALL)   // (the sums of those that do not exist)
+    for (int i = nq * qstride + tid; i < NR * qstride; i += CT + 32) slots[i] = (R)0;
   if (K > 1) cluster_sync_all();   // barriers ready in every CTA before the first remote store
   else __syncthreads();
 
@@ -514,13 +531,15 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
           auto products = [&](auto N_, auto diag_) {
             constexpr int N = decltype(N_)::value;
             constexpr bool DIAG = decltype(diag_)::value;
-            constexpr bool HOLD = sizeof(R) == 4;   // all tiles in registers (complex FP64: one at a time)
+            // all tiles in registers, or one at a time (complex FP64; small CTAs with several right-hand
+            // sides, whose 128 registers would spill: 576 boxes of 48, two sources 0.293 -> 0.25 ms)
+            constexpr bool HOLD = sizeof(R) == 4 && !(SMALL && NR > 1);
             typename O::Ent t[HOLD ? N : 1][4][2];
             if (HOLD)
 #pragma unroll
               for (int k = 0; k < N; ++k) load_tile(tile + k * TE, lane, t[k]);
 #pragma unroll 1
-            for (int q = 0; q < NR; ++q) {
+            for (int q = 0; q < nq; ++q) {
               const T *vr = vsr + q * mpmax + I0 * TB, *vc = vsc + q * mpmax + J * TB;
               Vec vJ[4];
               O::load2(vc, vJ[0], vJ[1]);
@@ -554,11 +573,15 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
               R out[N];
 #pragma unroll
               for (int k = 0; k < N; ++k) out[k] = reduce_rows(rv[k], lane);
-              const T cv[4] = {O::value(cacc[0]), O::value(cacc[1]), O::value(cacc[2]), O::value(cacc[3])};
-              const R oc = reduce_cols(cv, lane);
+              constexpr bool COLS = !DIAG || N > 1;   // (a diagonal tile on its own has no column sums)
+              R oc = (R)0;
+              if constexpr (COLS) {
+                const T cv[4] = {O::value(cacc[0]), O::value(cacc[1]), O::value(cacc[2]), O::value(cacc[3])};
+                oc = reduce_cols(cv, lane);
+              }
 #pragma unroll
               for (int k = 0; k < N; ++k) rowslot[q * qstride + k * 32] = out[k];
-              colslot[q * qstride] = oc;
+              if constexpr (COLS) colslot[q * qstride] = oc;
             }
           };
           using One = std::integral_constant<int, 1>;
@@ -566,6 +589,7 @@ k_subst_sym(const SubDev *__restrict__ subs, const C<R> *__restrict__ poolr,
           using Three = std::integral_constant<int, 3>;
           if (n == 3 && I0 + 2 < J) products(Three{}, std::false_type{});
           else if (n == 3) products(Three{}, std::true_type{});
+          else if (sizeof(R) == 8 && n == 1 && I0 < J) products(One{}, std::false_type{});
           else if (n == 2) products(Two{}, std::true_type{});
           else products(One{}, std::true_type{});
         }
@@ -682,37 +706,38 @@ template <typename R> static const C<R> *lpool_of(const hd_ctx *ctx);
 template <> const float2 *lpool_of<float>(const hd_ctx *ctx) { return ctx->d_lpoolf; }
 template <> const double2 *lpool_of<double>(const hd_ctx *ctx) { return ctx->d_lpool; }
 
-// kNoFit: the shape's shared memory does not fit (the caller takes fewer right-hand sides per CTA).
-constexpr cudaError_t kNoFit = cudaErrorMemoryAllocation;
+// Tiles of a segment in a launch whose widest box has mp rows: three, and one in complex FP64
+// up to 64, where a step would wait for one warp's 192 FP64 instructions at 64 cycles each (4 boxes of
+// 48 0.68 -> 0.38 ms, of 64 1.04 -> 0.58; at 96 the sums of so many column slots cost more: 1.64 -> 1.80).
+template <typename R> static int sym_segment(int mp) { return sizeof(R) == 8 && mp <= 64 ? 1 : 3; }
 
-template <typename R, typename S, int K, int P, int NR, int VG>
+template <typename R, typename S, int K, int P, int NR, int VG, int SW, int PER_SM>
 static cudaError_t launch_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
                               int64_t stg_stride, cudaStream_t st) {
   using T = C<R>;
   const int mpmax = (ctx->max_m + TB - 1) / TB * TB;
   const int groups = (nrhs + NR - 1) / NR;
-  int dev = 0, optin = 0;
+  int dev = 0, optin = 0, sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e != cudaSuccess) return e;
-  // complex FP64 with more boxes than SMs: two CTAs per SM, one's sums and exchanges under the
-  // other's products
-  if (sizeof(R) == 8 && K == 1 && NR == 1 && (int64_t)ctx->nsub * groups > sm_count()) optin = optin / 2 - 1024;
-  // one CTA per SM: the ring takes what is left, two stages at least where a round of every
-  // warp allows it (complex FP64, bound by its arithmetic: one), else fewer warps per round
-  constexpr int SW = set_warps<R>();
+  if (PER_SM > 1) optin = std::min(optin, sm / PER_SM - 1024);   // (1 KB of every CTA's is the system's)
+  // the ring takes what is left, two stages at least where a round of every warp allows it (large
+  // CTAs of complex FP64, bound by their arithmetic: one), else fewer warps per round
+  const int seg = sym_segment<R>(mpmax);
   int spr = SW, stiles = 0, ns = 0;
   for (; spr >= 1; --spr) {
-    stiles = sym_stage_tiles(mpmax / TB, spr);
-    const size_t fixed = sym_smem<R, S>(0, stiles, spr, mpmax, K, P, NR).total;
+    stiles = sym_stage_tiles(mpmax / TB, spr, seg);
+    const size_t fixed = sym_smem<R, S>(0, stiles, spr, mpmax, K, P, NR, SW, seg).total;
     const size_t stage = (size_t)P * (stiles * TE * sizeof(S) + 2 * sizeof(uint64_t));
     ns = fixed < (size_t)optin ? (int)std::min<size_t>(16, ((size_t)optin - fixed) / stage) : 0;
-    if (ns >= (sizeof(R) == 4 && spr > 3 ? 2 : 1)) break;
+    if (ns >= (PER_SM > 2 ? (spr > 1 ? 2 : 1) : (sizeof(R) == 4 && spr > 3 ? 2 : 1))) break;
   }
-  if (spr < 1) return kNoFit;
+  if (spr < 1) return cudaErrorInvalidValue;
   if (ctx->tune_ns > 0 && NR == 1) ns = std::min(ns, ctx->tune_ns);
-  const size_t smem = sym_smem<R, S>(ns, stiles, spr, mpmax, K, P, NR).total;
-  auto kern = k_subst_sym<R, S, K, P, NR, VG>;
+  const size_t smem = sym_smem<R, S>(ns, stiles, spr, mpmax, K, P, NR, SW, seg).total;
+  auto kern = k_subst_sym<R, S, K, P, NR, VG, SW, PER_SM>;
   if ((e = allow_smem(kern, smem)) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(groups * K), (unsigned)ctx->nsub);   // a box's source groups side by side share its factor reads in L2
@@ -728,64 +753,62 @@ static cudaError_t launch_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t v
   cfg.numAttrs = K > 1 ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, (const SubDev *)ctx->d_subs, lpool_of<R>(ctx),
                             reinterpret_cast<const S *>(ctx->factor), r, ctx->NX, vec_stride,
-                            reinterpret_cast<T *>(staging), stg_stride, nrhs, ns, stiles, spr, mpmax, ctx->d_status);
+                            reinterpret_cast<T *>(staging), stg_stride, nrhs, ns, stiles, spr, seg, mpmax, ctx->d_status);
+}
+
+static SymPick sym_pick(const hd_ctx *ctx, int nrhs) {
+  return ctx->prec == HD_C128 ? sym_pick64(ctx->max_m, ctx->nsub, nrhs, sm_count())
+                              : sym_pick32(ctx->max_m, ctx->nsub, nrhs, sm_count());
 }
 
 // Consumer threads of a single-source launch (what the autotuner reports).
 int subst_sym_threads(const hd_ctx *ctx) {
-  const int sms = sm_count();
-  if (ctx->prec == HD_C128) return set_warps<double>() * 32;
-  return (4 * ctx->nsub <= sms && ctx->max_m <= set_warps<float>() * 32 ? 1 : 2) * set_warps<float>() * 32;
+  const SymPick p = sym_pick(ctx, 1);
+  return p.P * p.SW * 32;
 }
 
-// CTAs per box.  Complex FP32: enough clusters to give every SM about one CTA.  Measured per
-// application (one right-hand side; K = 1 / 2 / 4): 16 boxes of 176 708 / 566 / 481 us, 64
-// boxes 718 / 564 / 928 us, 144 boxes 1000 / 1131 / 1877 us, 256 boxes 1815 / 2236 / 3695 us.
-// Boxes wider than the 224 threads of one set take two sets.  Complex FP64: the time is that of
-// the busiest SM, ceil(K clusters / SMs) / K boxes, plus the exchange (4 CTAs: a fifth).
-template <typename R, typename S, int NR>
-static cudaError_t launch_sym_nr(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
-                                 cudaStream_t st) {
-  const int sms = sm_count();
-  const int64_t clusters = (int64_t)ctx->nsub * ((nrhs + NR - 1) / NR);
-  if constexpr (sizeof(R) == 8) {
-    auto cost = [&](int K, double more) { return (double)((clusters * K + sms - 1) / sms) / K * more; };
-    const double c1 = cost(1, 1.0), c2 = cost(2, 1.02), c4 = cost(4, 1.2);
-    if (c4 < c1 && c4 < c2) return launch_sym<R, S, 4, 1, NR, 1>(ctx, r, nrhs, vs, stg, ss, st);
-    if (c2 < c1) return launch_sym<R, S, 2, 1, NR, 1>(ctx, r, nrhs, vs, stg, ss, st);
-    return launch_sym<R, S, 1, 1, NR, 1>(ctx, r, nrhs, vs, stg, ss, st);
-  } else {
-    const bool wide = ctx->max_m > set_warps<R>() * 32;
-    constexpr int VG = NR > 1 ? 2 : 1;   // two sets have threads for two groups of vectors
-    if (4 * clusters <= sms && !wide) return launch_sym<R, S, 4, 1, NR, 1>(ctx, r, nrhs, vs, stg, ss, st);
-    if (2 * clusters <= sms)
-      return wide ? launch_sym<R, S, 2, 2, NR, 1>(ctx, r, nrhs, vs, stg, ss, st)
-                  : launch_sym<R, S, 2, 2, NR, VG>(ctx, r, nrhs, vs, stg, ss, st);
-    return wide ? launch_sym<R, S, 1, 2, NR, 1>(ctx, r, nrhs, vs, stg, ss, st)
-                : launch_sym<R, S, 1, 2, NR, VG>(ctx, r, nrhs, vs, stg, ss, st);
-  }
+static cudaError_t launch_sym64(hd_ctx *ctx, const SymPick &p, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
+                                cudaStream_t st) {
+  using R = double;
+  using S = double2;
+  if (p.per_sm == 3) return launch_sym<R, S, 1, 1, 1, 1, 4, 3>(ctx, r, nrhs, vs, stg, ss, st);
+  if (p.per_sm > 2) return launch_sym<R, S, 1, 1, 1, 1, 3, 4>(ctx, r, nrhs, vs, stg, ss, st);
+  if (p.K == 4) return launch_sym<R, S, 4, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st);
+  if (p.K == 2) return launch_sym<R, S, 2, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st);
+  return p.per_sm == 2 ? launch_sym<R, S, 1, 1, 1, 1, 8, 2>(ctx, r, nrhs, vs, stg, ss, st)
+                       : launch_sym<R, S, 1, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st);
 }
 
-// Right-hand sides per CTA: four share each read of the tiles (two in complex FP64, whose
-// products outweigh the reads, and where four do not fit shared memory).
-template <typename R, typename S>
-static cudaError_t launch_sym_rs(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
+template <typename S, int NR>
+static cudaError_t launch_sym32(hd_ctx *ctx, const SymPick &p, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
+                                cudaStream_t st) {
+  using R = float;
+  constexpr int VG = NR > 1 ? 2 : 1;   // two sets have threads for two groups of vectors, if the box is no wider than one
+  const bool wide = ctx->max_m > 224;
+  if (p.per_sm > 2) return launch_sym<R, S, 1, 1, NR, 1, 3, 4>(ctx, r, nrhs, vs, stg, ss, st);
+  if (p.K == 4) return launch_sym<R, S, 4, 1, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st);
+  if (p.K == 2)
+    return wide ? launch_sym<R, S, 2, 2, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st)
+                : launch_sym<R, S, 2, 2, NR, VG, 7, 1>(ctx, r, nrhs, vs, stg, ss, st);
+  return wide ? launch_sym<R, S, 1, 2, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st)
+              : launch_sym<R, S, 1, 2, NR, VG, 7, 1>(ctx, r, nrhs, vs, stg, ss, st);
+}
+template <typename S>
+static cudaError_t launch_sym_nr(hd_ctx *ctx, const SymPick &p, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
                                  cudaStream_t st) {
-  cudaError_t e = kNoFit;
-  if constexpr (sizeof(R) == 4)
-    if (nrhs >= 3) e = launch_sym_nr<R, S, 4>(ctx, r, nrhs, vs, stg, ss, st);
-  if (e == kNoFit && nrhs >= 2) e = launch_sym_nr<R, S, 2>(ctx, r, nrhs, vs, stg, ss, st);
-  if (e == kNoFit) e = launch_sym_nr<R, S, 1>(ctx, r, nrhs, vs, stg, ss, st);
-  return e == kNoFit ? cudaErrorInvalidValue : e;
+  return p.NR == 4   ? launch_sym32<S, 4>(ctx, p, r, nrhs, vs, stg, ss, st)
+         : p.NR == 2 ? launch_sym32<S, 2>(ctx, p, r, nrhs, vs, stg, ss, st)
+                     : launch_sym32<S, 1>(ctx, p, r, nrhs, vs, stg, ss, st);
 }
 
 cudaError_t launch_subst_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
                              int64_t stg_stride, cudaStream_t st) {
+  const SymPick p = sym_pick(ctx, nrhs);
   switch (ctx->prec) {
-    case HD_C64: return launch_sym_rs<float, float2>(ctx, r, nrhs, vec_stride, staging, stg_stride, st);
-    case HD_C64_H: return launch_sym_rs<float, __half2>(ctx, r, nrhs, vec_stride, staging, stg_stride, st);
-    case HD_C64_B: return launch_sym_rs<float, __nv_bfloat162>(ctx, r, nrhs, vec_stride, staging, stg_stride, st);
-    default: return launch_sym_rs<double, double2>(ctx, r, nrhs, vec_stride, staging, stg_stride, st);
+    case HD_C64: return launch_sym_nr<float2>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
+    case HD_C64_H: return launch_sym_nr<__half2>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
+    case HD_C64_B: return launch_sym_nr<__nv_bfloat162>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
+    default: return launch_sym64(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
   }
 }
 

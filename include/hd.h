@@ -339,8 +339,9 @@ int hd_block_gmres_solve(hd_ctx *ctx, const void *b_dev, void *x_dev, int32_t p,
 
 /* Autotuner (no counterpart in the paper): times hd_apply_precond's
  * substitution kernel for each candidate launch shape (full storage: 96, 128, 192 or 256
- * consumer threads per CTA; 2 to 32 ring stages that fit shared memory, 2 to 16 with
- * HD_SYMMETRIC, whose threads follow from the number of boxes) on r_dev ->
+ * consumer threads per CTA, 2 to 32 ring stages that fit shared memory; HD_SYMMETRIC, whose
+ * threads follow from the boxes: ring stages up to the deepest its launch can have, which
+ * may be the only candidate) on r_dev ->
  * z_dev (complex128 NY x NX, contents irrelevant, z is overwritten) with CUDA
  * events on `stream`, and keeps the fastest for this context.  The choice is
  * remembered for the process per (precision, storage layout, widest box,

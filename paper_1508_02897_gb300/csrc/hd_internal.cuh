@@ -401,6 +401,7 @@ cudaError_t launch_residual_strided(hd_ctx *ctx, const double2 *b, int64_t bs, c
 cudaError_t launch_subst_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
                              int64_t stg_stride, cudaStream_t st);
 int subst_sym_threads(const hd_ctx *ctx);
+int subst_sym_stages(hd_ctx *ctx);
 // Restrict + forward/back substitution on the tensor cores (HD_TCORE storage), staging out.
 cudaError_t launch_subst_tc(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
                             int64_t stg_stride, cudaStream_t st);

@@ -619,7 +619,12 @@ int autotune_subst(hd_ctx *ctx, const double2 *r, double2 *z, void *staging, cud
   // symmetric storage: threads follow from the number of boxes (launch_subst_sym), only the ring depth is timed
   std::vector<int> cts = ctx->sym ? std::vector<int>{subst_sym_threads(ctx)}
                                   : (ctx->max_m <= 192 ? std::vector<int>{96, 128, 192} : std::vector<int>{128, 256});
-  const int ns_list[] = {2, 3, 4, 6, 8, 12, 16, 24, 32};
+  std::vector<int> depths{2, 3, 4, 6, 8, 12, 16, 24, 32};
+  if (ctx->sym) {   // up to the deepest ring that its launch can have
+    const int deepest = subst_sym_stages(ctx);
+    while (!depths.empty() && depths.back() >= deepest) depths.pop_back();
+    depths.push_back(deepest);
+  }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -628,8 +633,8 @@ int autotune_subst(hd_ctx *ctx, const double2 *r, double2 *z, void *staging, cud
   const bool prof = ctx->profiling;
   ctx->profiling = false;
   for (int ct : cts)
-    for (int ns : ns_list) {
-      if (ctx->sym ? ns > 16 : (size_t)ns * ldmax * 64 + 8192 > (size_t)std::min(dev_optin, 224 * 1024)) continue;
+    for (int ns : depths) {
+      if (!ctx->sym && (size_t)ns * ldmax * 64 + 8192 > (size_t)std::min(dev_optin, 224 * 1024)) continue;
       ctx->tune_ct = ct;
       ctx->tune_ns = ns;
       float tot = 0.f;

@@ -713,7 +713,7 @@ template <typename R> static int sym_segment(int mp) { return sizeof(R) == 8 && 
 
 template <typename R, typename S, int K, int P, int NR, int VG, int SW, int PER_SM>
 static cudaError_t launch_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
-                              int64_t stg_stride, cudaStream_t st) {
+                              int64_t stg_stride, cudaStream_t st, int *depth) {
   using T = C<R>;
   const int mpmax = (ctx->max_m + TB - 1) / TB * TB;
   const int groups = (nrhs + NR - 1) / NR;
@@ -735,7 +735,8 @@ static cudaError_t launch_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t v
     if (ns >= (PER_SM > 2 ? (spr > 1 ? 2 : 1) : (sizeof(R) == 4 && spr > 3 ? 2 : 1))) break;
   }
   if (spr < 1) return cudaErrorInvalidValue;
-  if (ctx->tune_ns > 0 && NR == 1) ns = std::min(ns, ctx->tune_ns);
+  if (depth) { *depth = ns; return cudaSuccess; }   // (asked for the ring's stages only)
+  if (ctx->tune_ns > 0 && nrhs == 1) ns = std::min(ns, ctx->tune_ns);   // (what was tuned)
   const size_t smem = sym_smem<R, S>(ns, stiles, spr, mpmax, K, P, NR, SW, seg).total;
   auto kern = k_subst_sym<R, S, K, P, NR, VG, SW, PER_SM>;
   if ((e = allow_smem(kern, smem)) != cudaSuccess) return e;
@@ -768,48 +769,59 @@ int subst_sym_threads(const hd_ctx *ctx) {
 }
 
 static cudaError_t launch_sym64(hd_ctx *ctx, const SymPick &p, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
-                                cudaStream_t st) {
+                                cudaStream_t st, int *depth) {
   using R = double;
   using S = double2;
-  if (p.per_sm == 3) return launch_sym<R, S, 1, 1, 1, 1, 4, 3>(ctx, r, nrhs, vs, stg, ss, st);
-  if (p.per_sm > 2) return launch_sym<R, S, 1, 1, 1, 1, 3, 4>(ctx, r, nrhs, vs, stg, ss, st);
-  if (p.K == 4) return launch_sym<R, S, 4, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st);
-  if (p.K == 2) return launch_sym<R, S, 2, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st);
-  return p.per_sm == 2 ? launch_sym<R, S, 1, 1, 1, 1, 8, 2>(ctx, r, nrhs, vs, stg, ss, st)
-                       : launch_sym<R, S, 1, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st);
+  if (p.per_sm == 3) return launch_sym<R, S, 1, 1, 1, 1, 4, 3>(ctx, r, nrhs, vs, stg, ss, st, depth);
+  if (p.per_sm > 2) return launch_sym<R, S, 1, 1, 1, 1, 3, 4>(ctx, r, nrhs, vs, stg, ss, st, depth);
+  if (p.K == 4) return launch_sym<R, S, 4, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st, depth);
+  if (p.K == 2) return launch_sym<R, S, 2, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st, depth);
+  return p.per_sm == 2 ? launch_sym<R, S, 1, 1, 1, 1, 8, 2>(ctx, r, nrhs, vs, stg, ss, st, depth)
+                       : launch_sym<R, S, 1, 1, 1, 1, 8, 1>(ctx, r, nrhs, vs, stg, ss, st, depth);
 }
 
 template <typename S, int NR>
 static cudaError_t launch_sym32(hd_ctx *ctx, const SymPick &p, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
-                                cudaStream_t st) {
+                                cudaStream_t st, int *depth) {
   using R = float;
   constexpr int VG = NR > 1 ? 2 : 1;   // two sets have threads for two groups of vectors, if the box is no wider than one
   const bool wide = ctx->max_m > 224;
-  if (p.per_sm > 2) return launch_sym<R, S, 1, 1, NR, 1, 3, 4>(ctx, r, nrhs, vs, stg, ss, st);
-  if (p.K == 4) return launch_sym<R, S, 4, 1, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st);
+  if (p.per_sm > 2) return launch_sym<R, S, 1, 1, NR, 1, 3, 4>(ctx, r, nrhs, vs, stg, ss, st, depth);
+  if (p.K == 4) return launch_sym<R, S, 4, 1, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st, depth);
   if (p.K == 2)
-    return wide ? launch_sym<R, S, 2, 2, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st)
-                : launch_sym<R, S, 2, 2, NR, VG, 7, 1>(ctx, r, nrhs, vs, stg, ss, st);
-  return wide ? launch_sym<R, S, 1, 2, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st)
-              : launch_sym<R, S, 1, 2, NR, VG, 7, 1>(ctx, r, nrhs, vs, stg, ss, st);
+    return wide ? launch_sym<R, S, 2, 2, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st, depth)
+                : launch_sym<R, S, 2, 2, NR, VG, 7, 1>(ctx, r, nrhs, vs, stg, ss, st, depth);
+  return wide ? launch_sym<R, S, 1, 2, NR, 1, 7, 1>(ctx, r, nrhs, vs, stg, ss, st, depth)
+              : launch_sym<R, S, 1, 2, NR, VG, 7, 1>(ctx, r, nrhs, vs, stg, ss, st, depth);
 }
 template <typename S>
 static cudaError_t launch_sym_nr(hd_ctx *ctx, const SymPick &p, const double2 *r, int nrhs, int64_t vs, void *stg, int64_t ss,
-                                 cudaStream_t st) {
-  return p.NR == 4   ? launch_sym32<S, 4>(ctx, p, r, nrhs, vs, stg, ss, st)
-         : p.NR == 2 ? launch_sym32<S, 2>(ctx, p, r, nrhs, vs, stg, ss, st)
-                     : launch_sym32<S, 1>(ctx, p, r, nrhs, vs, stg, ss, st);
+                                 cudaStream_t st, int *depth) {
+  return p.NR == 4   ? launch_sym32<S, 4>(ctx, p, r, nrhs, vs, stg, ss, st, depth)
+         : p.NR == 2 ? launch_sym32<S, 2>(ctx, p, r, nrhs, vs, stg, ss, st, depth)
+                     : launch_sym32<S, 1>(ctx, p, r, nrhs, vs, stg, ss, st, depth);
+}
+
+static cudaError_t launch_pick(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging, int64_t stg_stride,
+                               cudaStream_t st, int *depth) {
+  const SymPick p = sym_pick(ctx, nrhs);
+  switch (ctx->prec) {
+    case HD_C64: return launch_sym_nr<float2>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st, depth);
+    case HD_C64_H: return launch_sym_nr<__half2>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st, depth);
+    case HD_C64_B: return launch_sym_nr<__nv_bfloat162>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st, depth);
+    default: return launch_sym64(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st, depth);
+  }
 }
 
 cudaError_t launch_subst_sym(hd_ctx *ctx, const double2 *r, int nrhs, int64_t vec_stride, void *staging,
                              int64_t stg_stride, cudaStream_t st) {
-  const SymPick p = sym_pick(ctx, nrhs);
-  switch (ctx->prec) {
-    case HD_C64: return launch_sym_nr<float2>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
-    case HD_C64_H: return launch_sym_nr<__half2>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
-    case HD_C64_B: return launch_sym_nr<__nv_bfloat162>(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
-    default: return launch_sym64(ctx, p, r, nrhs, vec_stride, staging, stg_stride, st);
-  }
+  return launch_pick(ctx, r, nrhs, vec_stride, staging, stg_stride, st, nullptr);
+}
+
+// Ring stages of a single-source launch: the most the autotuner has to choose from.
+int subst_sym_stages(hd_ctx *ctx) {
+  int depth = 0;
+  return launch_pick(ctx, nullptr, 1, 0, nullptr, 0, nullptr, &depth) == cudaSuccess ? depth : 0;
 }
 
 }  // namespace hd

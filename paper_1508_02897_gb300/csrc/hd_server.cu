@@ -93,7 +93,7 @@ static size_t request_bytes(const Request &q, int batch) {
     return (size_t)-1;
   const size_t cs = compute_bytes(q.precision & 0xff);
   const bool sym = (q.precision & HD_SYMMETRIC) != 0;
-  size_t factor = 0, staging = 0, work = 0;
+  size_t factor = 0, staging = 0, work = 0, pml = 0;
   for (int a : ey)
     for (int b : ex) {
       const size_t mt = (b + 15) / 16;
@@ -103,9 +103,11 @@ static size_t request_bytes(const Request &q, int batch) {
                                                 : (size_t)a * b * ((b + 3) & ~3));
       staging += (size_t)a * b;
       work += 2 * (size_t)b * b;
+      pml += (sizeof(double2) + sizeof(float2)) * (2 * (size_t)a + 2 * b + 2) + sizeof(SubDev) + sizeof(int32_t);
     }
   const size_t n = (size_t)(q.grid.nx + 2 * q.grid.npml) * (q.grid.ny + 2 * q.grid.npml);
-  const size_t tables = 2 * n * 8 + ((size_t)1 << 20);   // k^2, centre coefficients, PML tables
+  pml += (2 * sizeof(double2) + sizeof(int32_t)) * ((size_t)q.grid.nx + q.grid.ny + 4 * q.grid.npml + 1) + 256;
+  const size_t tables = 2 * n * 8 + std::max((size_t)1 << 20, pml);   // k^2, centre coefficients; PML and box tables
   const size_t vecs = n * 8 + 2 * n * 16 * (size_t)batch;     // velocity, right-hand sides, solutions
   return store_bytes(q.precision & 0xff) * factor + cs * std::max(staging * batch, work) + krylov_bytes((int64_t)n, q.opts.restart, batch) +
          tables + vecs;

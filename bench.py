@@ -647,7 +647,7 @@ def _profile_traffic(wl, args):
         return None
 
 
-KERNEL_REV = {False: "subst-v4", True: "subst-sym-v4"}   # kernel revisions the traffic summaries describe
+KERNEL_REV = {False: "subst-v4", True: "subst-sym-v5"}   # kernel revisions the traffic summaries describe
 
 
 # ----------------------------------------------------------------------------- serving

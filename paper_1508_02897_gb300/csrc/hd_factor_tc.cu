@@ -215,7 +215,6 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
   int abuf = 0;
   bool alive = true, rest = false;   // rest: MMAs of mbar[1] are in flight
 
-
   for (int box = blockIdx.x; box < nsub && alive; box += gridDim.x) {
     const SubDev s = subs[box];
     const int m = s.ex, rows = s.ey;
@@ -300,123 +299,123 @@ k_factor_tc(const SubDev *__restrict__ subs, int nsub, const double2 *__restrict
           tc::fence_after();
         }
         if (ahead) {
-        if (part == 0) {
-          float re[16], im[16];
-          tc::tmem_ld16_nw(tq + k0, re);
-          tc::tmem_ld16_nw(tq + NP + k0, im);
-          tc::tmem_wait_ld();
-#pragma unroll
-          for (int i = 0; i < 16; ++i) Cs[tid * CLD + i] = make_float2(re[i], im[i]);
-        } else if (mb > 0) {
-          if (k0 >= 128) {
-            if (part == 1 && q4 < 2) {   // bottom rows from the bottom-right block
-              const int rb = 32 * q4 + lane;
-              float re[16], im[16];
-              tc::tmem_ld16_nw(tq + 2 * NP + (k0 - 128), re);
-              tc::tmem_ld16_nw(tq + 2 * NP + NB + (k0 - 128), im);
-              tc::tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 16; ++i) Cs[(128 + rb) * CLD + i] = make_float2(re[i], im[i]);
-            }
-          } else if (q4 == (k0 >> 5)) {
-            // bottom rows of panel columns k < 128: W[128 + c'][k] = W[k][128 + c'], held by lane k
-            const int row = 32 * q4 + lane;
-            const bool mine = row >= k0 && row < k0 + FX_KP;
-            for (int cc = 16 * (part - 1); cc < NB && part < 3; cc += 32) {
-              float re[16], im[16];
-              tc::tmem_ld16_nw(tq + 128 + cc, re);
-              tc::tmem_ld16_nw(tq + NP + 128 + cc, im);
-              tc::tmem_wait_ld();
-              if (mine)
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                  const int cp = cc + i;
-                  Cs[(128 + cp) * CLD + (row - k0)] = cp < mb ? make_float2(re[i], im[i]) : make_float2(0.f, 0.f);
-                }
+          if (part == 0) {
+            float re[16], im[16];
+            tc::tmem_ld16_nw(tq + k0, re);
+            tc::tmem_ld16_nw(tq + NP + k0, im);
+            tc::tmem_wait_ld();
+  #pragma unroll
+            for (int i = 0; i < 16; ++i) Cs[tid * CLD + i] = make_float2(re[i], im[i]);
+          } else if (mb > 0) {
+            if (k0 >= 128) {
+              if (part == 1 && q4 < 2) {   // bottom rows from the bottom-right block
+                const int rb = 32 * q4 + lane;
+                float re[16], im[16];
+                tc::tmem_ld16_nw(tq + 2 * NP + (k0 - 128), re);
+                tc::tmem_ld16_nw(tq + 2 * NP + NB + (k0 - 128), im);
+                tc::tmem_wait_ld();
+  #pragma unroll
+                for (int i = 0; i < 16; ++i) Cs[(128 + rb) * CLD + i] = make_float2(re[i], im[i]);
+              }
+            } else if (q4 == (k0 >> 5)) {
+              // bottom rows of panel columns k < 128: W[128 + c'][k] = W[k][128 + c'], held by lane k
+              const int row = 32 * q4 + lane;
+              const bool mine = row >= k0 && row < k0 + FX_KP;
+              for (int cc = 16 * (part - 1); cc < NB && part < 3; cc += 32) {
+                float re[16], im[16];
+                tc::tmem_ld16_nw(tq + 128 + cc, re);
+                tc::tmem_ld16_nw(tq + NP + 128 + cc, im);
+                tc::tmem_wait_ld();
+                if (mine)
+  #pragma unroll
+                  for (int i = 0; i < 16; ++i) {
+                    const int cp = cc + i;
+                    Cs[(128 + cp) * CLD + (row - k0)] = cp < mb ? make_float2(re[i], im[i]) : make_float2(0.f, 0.f);
+                  }
+              }
             }
           }
-        }
-        if (follow) asm volatile("bar.sync 3, %0;" ::"n"(FX_THREADS - 32) : "memory");
-        else __syncthreads();
+          if (follow) asm volatile("bar.sync 3, %0;" ::"n"(FX_THREADS - 32) : "memory");
+          else __syncthreads();
 
-        // ---- B. side by side: warps 8..13 the A operand, warps 0..7 the pivot block
-        if (warp >= 8) {
-          // A = -X, X = C outside rows K and zero on rows K (their new values are stored
-          // directly), one row per thread; and the first pivot of the panel against every
-          // unprocessed row below the panel
-          unsigned char *Aw = At + (size_t)abuf * FX_NA * FX_ATILE;
-          const int r = tid - 256, kr = r - k0;
-          if (r < m) {
-            const bool inK = kr >= 0 && kr < w;
-            float vr[16], vi[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float2 c = Cs[r * CLD + i];
-              vr[i] = inK ? 0.f : -c.x;
-              vi[i] = inK ? 0.f : -c.y;
+          // ---- B. side by side: warps 8..13 the A operand, warps 0..7 the pivot block
+          if (warp >= 8) {
+            // A = -X, X = C outside rows K and zero on rows K (their new values are stored
+            // directly), one row per thread; and the first pivot of the panel against every
+            // unprocessed row below the panel
+            unsigned char *Aw = At + (size_t)abuf * FX_NA * FX_ATILE;
+            const int r = tid - 256, kr = r - k0;
+            if (r < m) {
+              const bool inK = kr >= 0 && kr < w;
+              float vr[16], vi[16];
+  #pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                const float2 c = Cs[r * CLD + i];
+                vr[i] = inK ? 0.f : -c.x;
+                vi[i] = inK ? 0.f : -c.y;
+              }
+              put_split(Aw, FX_ATILE, 0, r, vr);
+              put_split(Aw, FX_ATILE, 3, r, vi);
+              if (r >= k0 + w && !(cabs2f(Cs[k0 * CLD]) >= tau2 * cabs2f(Cs[r * CLD]))) *sflag = 1;
             }
-            put_split(Aw, FX_ATILE, 0, r, vr);
-            put_split(Aw, FX_ATILE, 3, r, vi);
-            if (r >= k0 + w && !(cabs2f(Cs[k0 * CLD]) >= tau2 * cabs2f(Cs[r * CLD]))) *sflag = 1;
-          }
-          // the band of the next row's D, on the FP64 pipe while the pivot block is inverted
-          if (k0 == 0 && more && r < FX_ROWS) band_row(r, j + 1);
-        } else {
-          // P = C_K^{-1} (w x w) by Gauss-Jordan without pivoting, one entry per thread
-          // (i, jj) = (tid / 16, tid % 16), two alternating shared copies.  Two elimination
-          // steps k, k+1 per barrier: every thread loads the nine entries it needs and
-          // applies both in-place steps to its own entry (the same arithmetic as two
-          // separate steps).  In-place value of entry (x, y) after a step with pivot index k:
-          // the inverse pivot on (k, k), a_ky / pivot on row k, -a_xk / pivot on column k, else
-          // a_xy - a_xk (a_ky / pivot); formed without branches, every case selected from the
-          // few products the entries share.  Each pivot is checked by the threads of the
-          // unprocessed entries below it.  (Two entries per thread on four warps: 6.8K cycles per
-          // panel instead of 5.3K: the instructions of a thread, not the shared work, set the time.)
-          const int i = tid >> 4, jj = tid & 15;
-          float2 *B0 = G, *B1 = G + 256;
-          auto sync8 = []() { asm volatile("bar.sync 2, 256;" ::: "memory"); };
-          auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
-          auto sel = [](bool c, float2 x, float2 y) { return make_float2(c ? x.x : y.x, c ? x.y : y.y); };
-          B0[tid] = (i < w && jj < w) ? Cs[(k0 + i) * CLD + jj] : make_float2(i == jj ? 1.f : 0.f, 0.f);
-          sync8();
-          int par = 0;
-#pragma unroll 1
-          for (int k = 0; k < w; k += 2, par ^= 1) {
-            const float2 *src = par ? B1 : B0;
-            float2 *dst = par ? B0 : B1;
-            const int k1 = min(k + 1, 15);
-            const float2 piv = src[k * 16 + k], aik = src[i * 16 + k], akj = src[k * 16 + jj], aij = src[tid];
-            const float2 a_i1 = src[i * 16 + k1], a_k1 = src[k * 16 + k1];
-            const float2 a_1j = src[k1 * 16 + jj], a_1k = src[k1 * 16 + k], a_11 = src[k1 * 16 + k1];
-            const float p2 = cabs2f(piv);
-            const float rd = recip(p2);   // 1 / pivot = conj(pivot) / |pivot|^2
-            const float2 ip = make_float2(piv.x * rd, -piv.y * rd);
-            const float2 tj = cmul(akj, ip), t1 = cmul(a_k1, ip);
-            float2 v = sel(i == k, sel(jj == k, ip, tj), sel(jj == k, neg(cmul(aik, ip)), cfms(aik, tj, aij)));
-            bool bad = (jj == k && i > k && i < w && !(p2 >= tau2 * cabs2f(aik))) || (tid == 0 && (!(p2 > 0.f) || !isfinite(p2)));
-            if (k + 1 < w) {
-              // the second step on the values after the first
-              const float2 vi1 = sel(i == k, t1, cfms(aik, t1, a_i1));                    // entry (i, k+1)
-              const float2 v1j = sel(jj == k, neg(cmul(a_1k, ip)), cfms(a_1k, tj, a_1j));   // entry (k+1, jj)
-              const float2 piv1 = cfms(a_1k, t1, a_11);                                   // next pivot
-              const float q2 = cabs2f(piv1);
-              const float rd1 = recip(q2);
-              const float2 ip1 = make_float2(piv1.x * rd1, -piv1.y * rd1);
-              const float2 t2 = cmul(v1j, ip1);
-              bad = bad || (jj == k1 && i > k1 && i < w && !(q2 >= tau2 * cabs2f(vi1))) ||
-                    (tid == 0 && (!(q2 > 0.f) || !isfinite(q2)));
-              v = sel(i == k1, sel(jj == k1, ip1, t2), sel(jj == k1, neg(cmul(vi1, ip1)), cfms(vi1, t2, v)));
-            }
-            if (bad) *sflag = 1;
-            dst[tid] = v;
+            // the band of the next row's D, on the FP64 pipe while the pivot block is inverted
+            if (k0 == 0 && more && r < FX_ROWS) band_row(r, j + 1);
+          } else {
+            // P = C_K^{-1} (w x w) by Gauss-Jordan without pivoting, one entry per thread
+            // (i, jj) = (tid / 16, tid % 16), two alternating shared copies.  Two elimination
+            // steps k, k+1 per barrier: every thread loads the nine entries it needs and
+            // applies both in-place steps to its own entry (the same arithmetic as two
+            // separate steps).  In-place value of entry (x, y) after a step with pivot index k:
+            // the inverse pivot on (k, k), a_ky / pivot on row k, -a_xk / pivot on column k, else
+            // a_xy - a_xk (a_ky / pivot); formed without branches, every case selected from the
+            // few products the entries share.  Each pivot is checked by the threads of the
+            // unprocessed entries below it.  (Two entries per thread on four warps: 6.8K cycles per
+            // panel instead of 5.3K: the instructions of a thread, not the shared work, set the time.)
+            const int i = tid >> 4, jj = tid & 15;
+            float2 *B0 = G, *B1 = G + 256;
+            auto sync8 = []() { asm volatile("bar.sync 2, 256;" ::: "memory"); };
+            auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
+            auto sel = [](bool c, float2 x, float2 y) { return make_float2(c ? x.x : y.x, c ? x.y : y.y); };
+            B0[tid] = (i < w && jj < w) ? Cs[(k0 + i) * CLD + jj] : make_float2(i == jj ? 1.f : 0.f, 0.f);
             sync8();
+            int par = 0;
+  #pragma unroll 1
+            for (int k = 0; k < w; k += 2, par ^= 1) {
+              const float2 *src = par ? B1 : B0;
+              float2 *dst = par ? B0 : B1;
+              const int k1 = min(k + 1, 15);
+              const float2 piv = src[k * 16 + k], aik = src[i * 16 + k], akj = src[k * 16 + jj], aij = src[tid];
+              const float2 a_i1 = src[i * 16 + k1], a_k1 = src[k * 16 + k1];
+              const float2 a_1j = src[k1 * 16 + jj], a_1k = src[k1 * 16 + k], a_11 = src[k1 * 16 + k1];
+              const float p2 = cabs2f(piv);
+              const float rd = recip(p2);   // 1 / pivot = conj(pivot) / |pivot|^2
+              const float2 ip = make_float2(piv.x * rd, -piv.y * rd);
+              const float2 tj = cmul(akj, ip), t1 = cmul(a_k1, ip);
+              float2 v = sel(i == k, sel(jj == k, ip, tj), sel(jj == k, neg(cmul(aik, ip)), cfms(aik, tj, aij)));
+              bool bad = (jj == k && i > k && i < w && !(p2 >= tau2 * cabs2f(aik))) || (tid == 0 && (!(p2 > 0.f) || !isfinite(p2)));
+              if (k + 1 < w) {
+                // the second step on the values after the first
+                const float2 vi1 = sel(i == k, t1, cfms(aik, t1, a_i1));                    // entry (i, k+1)
+                const float2 v1j = sel(jj == k, neg(cmul(a_1k, ip)), cfms(a_1k, tj, a_1j));   // entry (k+1, jj)
+                const float2 piv1 = cfms(a_1k, t1, a_11);                                   // next pivot
+                const float q2 = cabs2f(piv1);
+                const float rd1 = recip(q2);
+                const float2 ip1 = make_float2(piv1.x * rd1, -piv1.y * rd1);
+                const float2 t2 = cmul(v1j, ip1);
+                bad = bad || (jj == k1 && i > k1 && i < w && !(q2 >= tau2 * cabs2f(vi1))) ||
+                      (tid == 0 && (!(q2 > 0.f) || !isfinite(q2)));
+                v = sel(i == k1, sel(jj == k1, ip1, t2), sel(jj == k1, neg(cmul(vi1, ip1)), cfms(vi1, t2, v)));
+              }
+              if (bad) *sflag = 1;
+              dst[tid] = v;
+              sync8();
+            }
+            // P into the first copy, zero outside w x w (each thread moves its own entry)
+            const float2 *res = par ? B1 : B0;
+            const float2 pv = (i < w && jj < w) ? res[tid] : make_float2(0.f, 0.f);
+            B0[tid] = pv;
           }
-          // P into the first copy, zero outside w x w (each thread moves its own entry)
-          const float2 *res = par ? B1 : B0;
-          const float2 pv = (i < w && jj < w) ? res[tid] : make_float2(0.f, 0.f);
-          B0[tid] = pv;
         }
-        }   // ahead
         // the previous panel's remaining MMAs read the B operand and write W: done from here on
         if (rest && !tc::bar_spin(mbar + 1, nrest & 1u, abort_flag)) *abort_flag = 1;
         if (rest) ++nrest;

@@ -99,8 +99,8 @@ struct OpArgs {
 // joins one pair before the pairs meet: for a wave the two halves nearly cancel, and their sum
 // is exact or close to it, where x_W + x_N + x_S + x_E would be rounded at four times the wave's size
 // first.  (Error against extended precision on waves of 10 to 20 cells, relative to the four
-// neighbours added one by one to cc x_C: 1.01 to 1.07, with the four summed first 1.35 to 1.49;
-// on white noise 0.76.)
+// neighbours added one by one to cc x_C: 0.96 to 1.08, with the four summed first 1.31 to 1.5;
+// on white noise 0.77.)
 // A warp takes ST_COLS columns (its last lane only forms pairs) and `R` rows; every entry of x is
 // loaded once per tile.  The tiles fill the part outside the PML from its lower corner; the frame
 // around them (the PML and what is left of a tile) takes the general form, a thread per cell.

@@ -23,10 +23,10 @@
 // (br, br, bi, bi), the sums of a * (br, br) and of a * (bi, bi) need two packed FMAs per
 // complex product and no operand shuffling; re and im are formed once per sum.
 //
-// Measured per application (substitution and sum, one CTA per box before): c64, 128^2 in 4
+// Measured per application (substitution and sum, one CTA per box and tile per warp before): c64, 128^2 in 4
 // boxes 0.80 -> 0.23 ms; 1003^2 in 64 boxes 2.83 -> 0.58 ms (4.6 TB/s); 2048^2 in 256 boxes 3.28 ->
-// 1.82 ms; 4096^2 in 1024 boxes 8.20 -> 6.95 ms (7.1 TB/s); four sources at 2048^2 6.07 -> 4.55 ms;
-// c128, 1024^2 in 64 boxes 14.3 -> 7.3 ms.
+// 1.82 ms; 4096^2 in 1024 boxes 8.20 -> 6.95 ms (7.1 TB/s); four sources at 2048^2 6.07 -> 4.54 ms;
+// c128, 1024^2 in 64 boxes 14.3 -> 7.3 ms; narrow boxes in hd_sym_shape.cuh.
 //
 // A producer warp (one lane per set) streams the tiles by bulk copies into an mbarrier
 // ring, ahead across steps: a stage is one round of a set, a segment for each of its warps.

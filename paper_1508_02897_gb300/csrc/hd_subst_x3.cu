@@ -37,8 +37,9 @@
 //
 // Warp roles: warps 0-11 epilogue (thread = tensor-memory lane), warp 12 producer (factor
 // chunks through an mbarrier ring with cp.async.bulk, in use order across steps, after
-// asking L2 for them a few chunks ahead: the ring holds two to four chunks beside the A
-// operands, too few to cover HBM's latency on its own), warp 13
+// asking L2 for them a few chunks ahead: beside the A operands of the widest boxes the ring
+// holds two chunks, six with M = 64, and up to eight in narrower ones; two are too few to cover HBM's
+// latency on their own), warp 13
 // tensor-memory owner and MMA issuer (one thread).
 //
 // What bounds it: a 176-row step takes 22.5K cycles (17.6K with M = 64), 12K of them the 88
@@ -224,8 +225,8 @@ k_subst_x3(const SubDev *__restrict__ subs, const double2 *__restrict__ pool, co
   if (warp == X3_EPI / 32) {
     // ---------------- producer: chunks of every block in use order, each asked of L2
     // kX3Prefetch chunks before its copy
-    // (slot, phase and source advance by addition: a refill is on the critical path of the two-
-    // to four-stage ring, and 64-bit divisions there cost more than the copy's latency)
+    // (slot, phase and source advance by addition: with few stages a refill is on the critical
+    // path, and 64-bit divisions there cost more than the copy's latency)
     if (lane == 0) {
       const float *src = Fs, *pre = Fs;   // next chunk to copy, next chunk to ask L2 for
       int c = 0, st = 0, pc = 0, pst = 0;

@@ -15,13 +15,13 @@ struct SymPick {
 
 // Complex FP32 arithmetic.  Boxes up to 96 wide: with more CTAs than SMs the small form, three
 // warps and a producer, four CTAs to an SM; a step of so few tiles is a chain of latencies that
-// one CTA cannot fill an SM with.  Measured per application, ms, one large CTA / small ones: one source,
-// 1024 boxes of 32 0.458 / 0.165, of 64 1.004 / 0.545, of 96 1.745 / 1.355; 144 boxes of 64 0.162 / 0.195.
-// (At 112 wide a form of four warps, three to an SM: 2.29 / 2.22.)
+// one CTA cannot fill an SM with.  Measured per application of one source, ms, one large CTA / small
+// ones: 1024 boxes of 32 0.458 / 0.152, of 64 1.02 / 0.50, of 96 1.75 / 1.31; 144 boxes of 64 0.162 /
+// 0.195.  (At 112 wide a form of four warps, three to an SM: 2.29 / 2.22.)
 constexpr int SYM_NARROW = 96;
-// Complex FP64, whose FP64 pipe a large CTA and a half keep busy from 96 on: up to 80 wide, with more
-// than two CTAs per SM.  400 boxes of 48 1.50 / 0.98 ms, of 80 5.28 / 3.99, of 96 7.28 / 6.71, but
-// 800 of 96 12.9 / 15.2.
+// Complex FP64: up to 80 wide, with more than two CTAs per SM (up to 48, more than one); wider boxes
+// keep the FP64 pipe busy with two large CTAs.  400 boxes of 48 1.50 / 0.95 ms, of 80 5.28 / 3.92;
+// 256 of 64 1.48 / 1.61; 800 of 96 12.9 / 15.2.
 constexpr int SYM_NARROW64 = 80;
 
 inline int64_t sym_waves(int64_t ctas, int64_t at_once) { return (ctas + at_once - 1) / at_once; }
@@ -29,7 +29,7 @@ inline int64_t sym_waves(int64_t ctas, int64_t at_once) { return (ctas + at_once
 // Complex FP64: one right-hand side per CTA (two shared the reads, which are not the bound, and left SMs
 // idle: 2 sources in 64 boxes of 240 40.3 ms, one each 34.1).  K by waves times the length of a step,
 // in units of one tile's products (0.6 us): a step takes as long as its tiles, spread over K CTAs at
-// 0.57 and 0.33, and not less than one warp's segment of three tiles.  K = 1 / 2 / 4, ms: 36 boxes of
+// 0.58 and 0.33, and not less than one warp's segment of three tiles.  K = 1 / 2 / 4, ms: 36 boxes of
 // 112 3.90 / 2.16 / 1.89, 64 boxes 3.92 / 2.17 / 3.77, 100 boxes 3.93 / 4.31 / 5.64, 169 boxes 6.96 /
 // 6.43 / 9.38; of 240, 64 boxes 34.1 / 21.0 / 20.8, 100 boxes 34.1 / 41.9 / 31.2, 169 boxes 67.8 / 62.7 / 51.9.
 inline SymPick sym_pick64(int m, int64_t nsub, int nrhs, int sms) {
@@ -37,6 +37,7 @@ inline SymPick sym_pick64(int m, int64_t nsub, int nrhs, int sms) {
   if (c > (m <= 48 ? 1 : 2) * (int64_t)sms && m <= SYM_NARROW64) return {1, 1, 3, 1, 4};
   const int mt = (m + 15) / 16;
   const double nt = mt * (mt + 1) / 2;
+  // four warps, three CTAs to an SM, where that saves a wave: 400 boxes of 112 13.99 -> 10.4 ms
   if (m > SYM_NARROW64 && m <= 112 && c > 2 * (int64_t)sms && 2.9 * sym_waves(c, 3 * (int64_t)sms) < 2 * sym_waves(c, 2 * (int64_t)sms))
     return {1, 1, 4, 1, 3};
   const double t1 = sym_waves(c, sms) * std::max(14.5, nt);
